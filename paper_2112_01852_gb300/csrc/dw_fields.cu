@@ -15,24 +15,38 @@ namespace dw {
 // slices per CTA through shared memory: the internal side of the chunk is one
 // contiguous run of vecs (coalesced 16-byte accesses, 8-byte at FP16), the
 // canonical side is kSC x 12 consecutive complex128 per site (coalesced
-// 16-byte accesses); the transpose itself happens in shared memory, one FP64
-// real per (site, slice, internal real I), rows padded to an odd length.
+// 16-byte accesses).  The staging array holds the canonical complex128 records,
+// one row per site padded by one record to an odd count, so the 16-byte accesses of
+// both sides are free of bank conflicts.
 constexpr int kSC = 4;        // slices per CTA
 constexpr int kXposeTPB = 128;
-constexpr int kLaneStride = kSC * 24 + 1;  // doubles per site row of the staging array
+constexpr int kRow = kSC * 12 + 1;  // complex128 records per site row of the staging array
 
-// internal real of the real part of canonical complex kk (spin*3 + colour);
-// the imaginary part is the internal real P::IM further on.  Spin-pair quads
-// (Re j0, Re j1, Im j0, Im j1); interleaved-complex quads (CPLX, the layout
-// ablation) (Re j0, Im j0, Re j1, Im j1).
+// One quad (spin pair j0, j1 of one colour and chirality half) <-> its two
+// canonical complex values.  Spin-pair quads (Re j0, Re j1, Im j0, Im j1);
+// interleaved-complex quads (CPLX, the layout ablation) (Re j0, Im j0, Re j1, Im j1).
 template <class P>
-__device__ __forceinline__ int internal_re(int kk) {
-  const int spin = kk / 3, c = kk % 3;
-  return (spin >> 1) * 12 + c * 4 + (spin & 1) * (P::CPLX ? 2 : 1);
+__device__ __forceinline__ void quad_from_complex(typename P::vec *d, double2 a, double2 b) {
+  double r[4];
+  if (P::CPLX) {
+    r[0] = a.x; r[1] = a.y; r[2] = b.x; r[3] = b.y;
+  } else {
+    r[0] = a.x; r[1] = b.x; r[2] = a.y; r[3] = b.y;
+  }
+#pragma unroll
+  for (int w = 0; w < 4 / P::R; ++w)
+    d[w * kPlaneStride] = narrow_from_f64(r + w * P::R, (typename P::vec *)nullptr);
 }
 template <class P>
-__host__ __device__ constexpr int im_offset() {
-  return P::CPLX ? 1 : 2;
+__device__ __forceinline__ void quad_to_complex(double2 &a, double2 &b,
+                                                const typename P::vec (&v)[4 / P::R]) {
+  typename P::C r[4];
+#pragma unroll
+  for (int w = 0; w < 4 / P::R; ++w) widen(v[w], r + w * P::R);
+  double d[4];
+  f64_from_f32(d, r);
+  a = P::CPLX ? make_double2(d[0], d[1]) : make_double2(d[0], d[2]);
+  b = P::CPLX ? make_double2(d[2], d[3]) : make_double2(d[1], d[3]);
 }
 
 template <class P>
@@ -40,33 +54,44 @@ __global__ void __launch_bounds__(kXposeTPB) pack_kernel(typename P::vec *dst,
                                                          const double2 *src, int V4, int Ls,
                                                          long long rhs_stride, long long V5) {
   constexpr int NP = 24 / P::R;
-  __shared__ double sm[32 * kLaneStride];
+  __shared__ double2 sm[32 * kRow];
   const int nch = (Ls + kSC - 1) / kSC;
   const int blk = (int)(blockIdx.x / nch);
   const int s0 = (int)(blockIdx.x % nch) * kSC;
   const int sc = min(kSC, Ls - s0);
   const int rhs = blockIdx.y;
+  const int nlane = min(32, V4 - blk * 32);  // padding lanes are never read or written
   // canonical -> staging: consecutive threads read consecutive complex128
-  const int nin = 32 * sc * 12;
-  for (int o = threadIdx.x; o < nin; o += kXposeTPB) {
-    const int lane = o / (sc * 12), rem = o % (sc * 12), sl = rem / 12, kk = rem % 12;
-    const int x4 = blk * 32 + lane;
-    if (x4 >= V4) continue;
-    const double2 v = __ldcs(src + ((long long)rhs * V5 + (long long)x4 * Ls + s0 + sl) * 12 + kk);
-    double *b = sm + lane * kLaneStride + sl * 24 + internal_re<P>(kk);
-    b[0] = v.x;
-    b[im_offset<P>()] = v.y;
+  const double2 *sp = src + ((long long)rhs * V5 + (long long)blk * 32 * Ls + s0) * 12;
+  if (sc == kSC && nlane == 32) {
+    double2 v[32 * kSC * 12 / kXposeTPB];  // all loads of the chunk in flight at once
+#pragma unroll
+    for (int i = 0; i < 32 * kSC * 12 / kXposeTPB; ++i) {
+      const int o = threadIdx.x + i * kXposeTPB;
+      const int lane = o / (kSC * 12), rem = o % (kSC * 12);
+      v[i] = __ldcs(sp + (long long)lane * Ls * 12 + rem);
+    }
+#pragma unroll
+    for (int i = 0; i < 32 * kSC * 12 / kXposeTPB; ++i) {
+      const int o = threadIdx.x + i * kXposeTPB;
+      sm[o / (kSC * 12) * kRow + o % (kSC * 12)] = v[i];
+    }
+  } else {
+    for (int o = threadIdx.x; o < nlane * sc * 12; o += kXposeTPB) {
+      const int lane = o / (sc * 12), rem = o % (sc * 12);
+      sm[lane * kRow + rem] = __ldcs(sp + (long long)lane * Ls * 12 + rem);
+    }
   }
   __syncthreads();
-  // staging -> internal: the chunk is one contiguous run of sc * NP * 32 vecs
+  // staging -> internal: the chunk is one contiguous run of sc * NP * 32 vecs; a
+  // warp writes one quad of one slice
   typename P::vec *dp = dst + rhs * rhs_stride + ((long long)blk * Ls + s0) * NP * 32;
-  for (int v = threadIdx.x; v < sc * NP * 32; v += kXposeTPB) {
-    const int lane = v & 31, q = (v >> 5) % NP, sl = (v >> 5) / NP;
-    if (blk * 32 + lane >= V4) continue;  // padding lanes are never written
-    double r[P::R];
-#pragma unroll
-    for (int w = 0; w < P::R; ++w) r[w] = sm[lane * kLaneStride + sl * 24 + q * P::R + w];
-    dp[v] = narrow_from_f64(r, (typename P::vec *)nullptr);
+  const int lane = threadIdx.x & 31;
+  if (lane >= nlane) return;
+  for (int v = threadIdx.x >> 5; v < sc * 6; v += kXposeTPB / 32) {
+    const int q = v % 6, sl = v / 6;  // quad: half * 3 + colour
+    const double2 *b = sm + lane * kRow + sl * 12 + (q / 3) * 6 + q % 3;
+    quad_from_complex<P>(dp + (sl * 6 + q) * (4 / P::R) * 32 + lane, b[0], b[3]);
   }
 }
 
@@ -75,34 +100,53 @@ __global__ void __launch_bounds__(kXposeTPB) unpack_kernel(double2 *dst,
                                                            const typename P::vec *src, int V4,
                                                            int Ls, long long rhs_stride,
                                                            long long V5) {
-  using C = typename P::C;
   constexpr int NP = 24 / P::R;
-  __shared__ double sm[32 * kLaneStride];
+  __shared__ double2 sm[32 * kRow];
   const int nch = (Ls + kSC - 1) / kSC;
   const int blk = (int)(blockIdx.x / nch);
   const int s0 = (int)(blockIdx.x % nch) * kSC;
   const int sc = min(kSC, Ls - s0);
   const int rhs = blockIdx.y;
-  // internal -> staging
+  const int nlane = min(32, V4 - blk * 32);
+  // internal -> staging: a warp reads one quad of one slice
   const typename P::vec *sp = src + rhs * rhs_stride + ((long long)blk * Ls + s0) * NP * 32;
-  for (int v = threadIdx.x; v < sc * NP * 32; v += kXposeTPB) {
-    const int lane = v & 31, q = (v >> 5) % NP, sl = (v >> 5) / NP;
-    if (blk * 32 + lane >= V4) continue;
-    C r[P::R];
-    load_vec<P>(r, sp + v);
+  const int lane = threadIdx.x & 31;
+  if (lane < nlane) {
+    constexpr int N = kSC * 6 / (kXposeTPB / 32);
+    typename P::vec r[N][4 / P::R];  // all loads of the chunk in flight at once
 #pragma unroll
-    for (int w = 0; w < P::R; ++w) sm[lane * kLaneStride + sl * 24 + q * P::R + w] = (double)r[w];
+    for (int i = 0; i < N; ++i) {
+      const int v = (threadIdx.x >> 5) + i * (kXposeTPB / 32);
+      if (v < sc * 6) {
+#pragma unroll
+        for (int w = 0; w < 4 / P::R; ++w) r[i][w] = __ldcs(sp + (v * (4 / P::R) + w) * 32 + lane);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const int v = (threadIdx.x >> 5) + i * (kXposeTPB / 32);
+      if (v < sc * 6) {
+        const int q = v % 6, sl = v / 6;
+        double2 *b = sm + lane * kRow + sl * 12 + (q / 3) * 6 + q % 3;
+        quad_to_complex<P>(b[0], b[3], r[i]);
+      }
+    }
   }
   __syncthreads();
   // staging -> canonical: consecutive threads write consecutive complex128
-  const int nout = 32 * sc * 12;
-  for (int o = threadIdx.x; o < nout; o += kXposeTPB) {
-    const int lane = o / (sc * 12), rem = o % (sc * 12), sl = rem / 12, kk = rem % 12;
-    const int x4 = blk * 32 + lane;
-    if (x4 >= V4) continue;
-    const double *b = sm + lane * kLaneStride + sl * 24 + internal_re<P>(kk);
-    __stcs(dst + ((long long)rhs * V5 + (long long)x4 * Ls + s0 + sl) * 12 + kk,
-           make_double2(b[0], b[im_offset<P>()]));
+  double2 *dp = dst + ((long long)rhs * V5 + (long long)blk * 32 * Ls + s0) * 12;
+  if (sc == kSC && nlane == 32) {
+#pragma unroll
+    for (int i = 0; i < 32 * kSC * 12 / kXposeTPB; ++i) {
+      const int o = threadIdx.x + i * kXposeTPB;
+      const int l = o / (kSC * 12), rem = o % (kSC * 12);
+      __stcs(dp + (long long)l * Ls * 12 + rem, sm[l * kRow + rem]);
+    }
+  } else {
+    for (int o = threadIdx.x; o < nlane * sc * 12; o += kXposeTPB) {
+      const int l = o / (sc * 12), rem = o % (sc * 12);
+      __stcs(dp + (long long)l * Ls * 12 + rem, sm[l * kRow + rem]);
+    }
   }
 }
 
@@ -152,48 +196,80 @@ int unpack_fermion(const FieldGeom &g, int prec, void *dst, const void *src, int
 // (link_off): all 18 reals at F64, the first two rows (12 reals) at F32 / F16.
 // A link U_mu(x) with x_mu = L_mu - 1 crosses the lattice edge and is
 // multiplied by bc[mu].
-template <class P>
-__device__ __forceinline__ void store_link(void *gauge, int mu, int x4, const double *u) {
-  typename P::vec *m = (typename P::vec *)gauge + link_off(x4, mu, P::NLV);
-#pragma unroll
-  for (int q = 0; q < P::NLV; ++q)
-    m[q * 32] = narrow_from_f64(u + q * P::R, (typename P::vec *)nullptr);
+// One CTA per 32-site block: its 32 x 4 links are 18 KB of consecutive canonical
+// memory and one contiguous run of each internal copy, so the block is read with
+// coalesced 16-byte loads into shared memory (one padded row of 4 x 18 reals per
+// site) and each copy is written with coalesced 16-byte (8-byte at FP16) stores.
+constexpr int kGaugeTPB = 128;
+constexpr int kGaugeRow = 4 * 9 + 1;  // complex128 records per site row (odd)
+
+// d with its sign bit flipped by f (the boundary factors are +-1)
+__device__ __forceinline__ double flip(double d, unsigned f) {
+  return __hiloint2double(__double2hiint(d) ^ (int)f, __double2loint(d));
 }
 
-__global__ void gauge_kernel(const double *U, int L0, int L1, int L2, int L3, int bc0, int bc1,
-                             int bc2, int bc3, void *g64, void *g32, void *g16) {
-  const long long V4 = (long long)L0 * L1 * L2 * L3;
-  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i >= 4 * V4) return;
-  const int x4 = (int)(i / 4);
-  const int mu = (int)(i % 4);
-  int c[4];
-  int rem = x4;
-  c[0] = rem % L0;
-  rem /= L0;
-  c[1] = rem % L1;
-  rem /= L1;
-  c[2] = rem % L2;
-  c[3] = rem / L2;
-  const int L[4] = {L0, L1, L2, L3};
-  const int bc[4] = {bc0, bc1, bc2, bc3};
-  const double f = (c[mu] == L[mu] - 1) ? (double)bc[mu] : 1.0;
-  double u[18];
-  const double *src = U + ((long long)x4 * 4 + mu) * 18;
+template <class P>
+__device__ __forceinline__ void store_links(void *gauge, int blk, int nlane, const double2 *sm,
+                                            const unsigned (*f)[4]) {
+  const int lane = threadIdx.x & 31;
+  if (lane >= nlane) return;
+  typename P::vec *m = (typename P::vec *)gauge + (long long)blk * 4 * P::NLV * 32;
+  for (int v = threadIdx.x >> 5; v < 4 * P::NLV; v += kGaugeTPB / 32) {
+    const int mu = v / P::NLV, q = v % P::NLV;
+    const double2 *s = sm + lane * kGaugeRow + mu * 9 + q * (P::R / 2);
+    const unsigned fm = f[lane][mu];
+    double r[P::R];
 #pragma unroll
-  for (int k = 0; k < 18; ++k) u[k] = f * src[k];
-  store_link<F64>(g64, mu, x4, u);
-  store_link<F32>(g32, mu, x4, u);
-  store_link<F16>(g16, mu, x4, u);
+    for (int k = 0; k < P::R / 2; ++k) {
+      r[2 * k] = flip(s[k].x, fm);
+      r[2 * k + 1] = flip(s[k].y, fm);
+    }
+    m[v * 32 + lane] = narrow_from_f64(r, (typename P::vec *)nullptr);
+  }
+}
+
+__global__ void __launch_bounds__(kGaugeTPB)
+    gauge_kernel(const double2 *U, int V4, int L0, int L1, int L2, int L3, int bc0, int bc1,
+                 int bc2, int bc3, void *g64, void *g32, void *g16) {
+  __shared__ double2 sm[32 * kGaugeRow];
+  __shared__ unsigned f[32][4];  // sign bit of the boundary factor of (site, mu)
+  const int blk = blockIdx.x;
+  const int nlane = min(32, V4 - blk * 32);
+  if ((int)threadIdx.x < nlane) {
+    int rem = blk * 32 + threadIdx.x;
+    const int L[4] = {L0, L1, L2, L3};
+    const int bc[4] = {bc0, bc1, bc2, bc3};
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      f[threadIdx.x][m] = (rem % L[m] == L[m] - 1 && bc[m] < 0) ? 0x80000000u : 0u;
+      rem /= L[m];
+    }
+  }
+  const double2 *src = U + (long long)blk * 32 * 36;
+  if (nlane == 32) {
+    double2 v[32 * 36 / kGaugeTPB];
+#pragma unroll
+    for (int i = 0; i < 32 * 36 / kGaugeTPB; ++i) v[i] = __ldcs(src + threadIdx.x + i * kGaugeTPB);
+#pragma unroll
+    for (int i = 0; i < 32 * 36 / kGaugeTPB; ++i) {
+      const int o = threadIdx.x + i * kGaugeTPB;
+      sm[o / 36 * kGaugeRow + o % 36] = v[i];
+    }
+  } else {
+    for (int o = threadIdx.x; o < nlane * 36; o += kGaugeTPB)
+      sm[o / 36 * kGaugeRow + o % 36] = src[o];
+  }
+  __syncthreads();
+  store_links<F64>(g64, blk, nlane, sm, f);
+  store_links<F32>(g32, blk, nlane, sm, f);
+  store_links<F16>(g16, blk, nlane, sm, f);
 }
 
 int load_gauge(const FieldGeom &g, const int bc[4], const void *U, void *const gauge[3],
                cudaStream_t st) {
-  const long long n = 4LL * g.V4;
-  const int tpb = 256;
-  gauge_kernel<<<(unsigned)((n + tpb - 1) / tpb), tpb, 0, st>>>(
-      (const double *)U, g.L[0], g.L[1], g.L[2], g.L[3], bc[0], bc[1], bc[2], bc[3], gauge[0],
-      gauge[1], gauge[2]);
+  gauge_kernel<<<(unsigned)(padded_v4(g.V4) / 32), kGaugeTPB, 0, st>>>(
+      (const double2 *)U, g.V4, g.L[0], g.L[1], g.L[2], g.L[3], bc[0], bc[1], bc[2], bc[3],
+      gauge[0], gauge[1], gauge[2]);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
