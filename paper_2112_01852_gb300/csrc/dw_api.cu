@@ -60,6 +60,42 @@ int ensure_buffer(void **buf, size_t *cap, size_t need) {
   return DW_OK;
 }
 
+PhiScratch::PhiScratch(dw_lattice *lat, int op, int prec, int nrhs, cudaStream_t st_) : st(st_) {
+  if (op != OP_D || prec != DW_F64 || lat->V5 * nrhs < kPhiPassMinSites) return;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return;
+  }
+  const size_t need = field_bytes(lat, prec, nrhs);
+  cudaMemPool_t pool;
+  {
+    std::lock_guard<std::mutex> g(lat->pool_lock);
+    if (!lat->pool) {
+      cudaMemPoolProps mp;
+      memset(&mp, 0, sizeof(mp));
+      mp.allocType = cudaMemAllocationTypePinned;
+      mp.location.type = cudaMemLocationTypeDevice;
+      mp.location.id = lat->device;
+      if (cudaMemPoolCreate(&lat->pool, &mp) != cudaSuccess) {
+        cudaGetLastError();
+        lat->pool = nullptr;
+        return;
+      }
+    }
+    if (need > lat->pool_keep) {
+      unsigned long long keep = need;
+      cudaMemPoolSetAttribute(lat->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+      lat->pool_keep = need;
+    }
+    pool = lat->pool;
+  }
+  if (cudaMallocFromPoolAsync(&p, need, pool, st) != cudaSuccess) {
+    cudaGetLastError();
+    p = nullptr;
+  }
+}
+
 // z-blocks of the traversal order: the fewest that keep the t-reuse window of
 // the input (2 * Lz/zblk planes x Ls slices) within ~20 MB of L2 (measured best
 // at 32^3 x 64 x 12: 4 z-blocks; 2 and 8 were slower).
@@ -142,12 +178,22 @@ long long dslash_ctas_per_rhs(const dw_lattice *lat, TileConfig t) {
 int run_dslash(dw_lattice *lat, int prec, int op, void *out, const void *in,
                const double *mf_host, int nrhs, cudaStream_t st, const TileConfig *force,
                const int *gate, int gate_stride, const void *halo_up, const void *halo_dn,
-               double *norm_partials, int t_begin, int t_count, const ResidualFuse *fuse) {
+               double *norm_partials, int t_begin, int t_count, const ResidualFuse *fuse,
+               void *phi) {
   const size_t rhs_bytes = field_bytes(lat, prec, 1);
   const int rs_prec = prec == DW_F64 ? DW_F64 : DW_F32;  // the residual's precision
   const size_t rs_rhs_bytes = field_bytes(lat, rs_prec, 1);
   if (fuse && op != OP_DDAG) return fail(DW_ERR_ARG, "the fused residual update is D^+ only");
   const size_t hrhs_bytes = halo_bytes(lat, prec, 1);
+  bool split = phi && op == OP_D && prec == DW_F64 && !halo_up && !halo_dn && !t_count;
+  if (split) {  // the plain hop has to take the CTA of the D tile
+    const TileConfig t = force ? *force : pick_tile(lat, prec, op, nrhs);
+    split = t.tx * (lat->Ls / t.spt / t.sgrp) <= dslash_max_threads(prec, OP_HOP_LOCAL, t.spt, 0);
+  }
+  if (split) {
+    const int rc = apply_phi(lat, prec, phi, in, false, mf_host, nrhs, st, gate, gate_stride);
+    if (rc) return rc;
+  }
   for (int r0 = 0; r0 < nrhs; r0 += kMaxRhsPerLaunch) {
     const int n = (nrhs - r0) < kMaxRhsPerLaunch ? (nrhs - r0) : kMaxRhsPerLaunch;
     DslashParams p;
@@ -179,7 +225,11 @@ int run_dslash(dw_lattice *lat, int prec, int op, void *out, const void *in,
     p.b = lat->b;
     p.c = lat->c;
     for (int r = 0; r < n; ++r) p.mf[r] = mf_host ? mf_host[r0 + r] : 0.0;
-    const TileConfig cfg = force ? *force : pick_tile(lat, prec, op, nrhs);
+    TileConfig cfg = force ? *force : pick_tile(lat, prec, op, nrhs);
+    if (split) {
+      p.in = (const char *)phi + (size_t)r0 * rhs_bytes;
+      cfg.variant = 0;  // same grid as the fused launch (FP64 variant 2 is variant 0 for D)
+    }
     p.rhs_outer = cfg.rhs_outer;
     p.norm_partials =
         norm_partials ? norm_partials + (size_t)r0 * dslash_ctas_per_rhs(lat, cfg) : nullptr;
@@ -202,7 +252,7 @@ int run_dslash(dw_lattice *lat, int prec, int op, void *out, const void *in,
                     "Dhop^+ only");
       rc = launch_dslash_cplx(p, op, cfg, st);
     } else {
-      rc = launch_dslash(p, prec, op, cfg, st);
+      rc = launch_dslash(p, prec, split ? OP_HOP_LOCAL : op, cfg, st);
     }
     if (rc == -2)
       return fail(DW_ERR_ARG, "unsupported tile (spt=%d, tx=%d, variant=%d, zblk=%d) for Ls=%d",
@@ -239,13 +289,20 @@ int apply_op(dw_lattice *lat, int op, void *out, const void *in, const double *m
     case DW_OP_DHOP: return run_dslash(lat, lat->prec, OP_DHOP, out, in, nullptr, nrhs, st, nullptr);
     case DW_OP_DHOP_DAG:
       return run_dslash(lat, lat->prec, OP_DHOP_DAG, out, in, nullptr, nrhs, st, nullptr);
-    case DW_OP_D: return run_dslash(lat, lat->prec, OP_D, out, in, mf, nrhs, st, nullptr);
+    case DW_OP_D: {
+      const PhiScratch phi(lat, OP_D, lat->prec, nrhs, st);
+      return run_dslash(lat, lat->prec, OP_D, out, in, mf, nrhs, st, nullptr, nullptr, 0, nullptr,
+                        nullptr, nullptr, 0, 0, nullptr, phi.p);
+    }
     case DW_OP_DDAG: return run_dslash(lat, lat->prec, OP_DDAG, out, in, mf, nrhs, st, nullptr);
     case DW_OP_DDAGD: {
       const size_t need = field_bytes(lat, lat->prec, nrhs);
       int rc = ensure_buffer(&lat->scratch, &lat->scratch_bytes, need);
       if (rc) return rc;
-      rc = run_dslash(lat, lat->prec, OP_D, lat->scratch, in, mf, nrhs, st, nullptr);
+      // (the phi scratch of the D pass is `out`, which D^+ writes last)
+      void *phi = lat->V5 * nrhs >= kPhiPassMinSites ? out : nullptr;
+      rc = run_dslash(lat, lat->prec, OP_D, lat->scratch, in, mf, nrhs, st, nullptr, nullptr, 0,
+                      nullptr, nullptr, nullptr, 0, 0, nullptr, phi);
       if (rc) return rc;
       return run_dslash(lat, lat->prec, OP_DDAG, out, lat->scratch, mf, nrhs, st, nullptr);
     }
@@ -339,6 +396,7 @@ void dw_destroy_lattice(dw_lattice *lat) {
   if (lat->dev_status) cudaFree(lat->dev_status);
   cg_release(lat);
   pipe_release(lat);
+  if (lat->pool) cudaMemPoolDestroy(lat->pool);
   delete lat;
 }
 

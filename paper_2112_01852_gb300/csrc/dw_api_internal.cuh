@@ -2,6 +2,7 @@
 #pragma once
 
 #include <map>
+#include <mutex>
 #include <tuple>
 #include <vector>
 
@@ -47,6 +48,11 @@ struct dw_lattice {
   std::map<std::tuple<int, int, int>, dw::TileConfig> tuned;
   // solver workspace (dw_cg_solve), created on first use
   dw::CGWork *cg;
+  // stream-ordered workspaces of single calls (PhiScratch): a pool of the lattice, so
+  // calls on several streams or threads each get their own block
+  std::mutex pool_lock;
+  cudaMemPool_t pool;
+  size_t pool_keep;  // bytes the pool keeps between calls (one workspace)
 };
 
 namespace dw {
@@ -74,11 +80,29 @@ int tune_tile(dw_lattice *lat, int prec, int op, int nrhs, cudaStream_t st, bool
 // (t_count 0: all).
 // `fuse` (optional, OP_DDAG only): the CG residual update of ResidualFuse in place
 // of storing out (out is then not written).
+// `phi` (optional): scratch of the input's size; an FP64 OP_D then forms phi there in
+// a pass of its own (same result bit for bit, fewer FP64 operations).
 int run_dslash(dw_lattice *lat, int prec, int op, void *out, const void *in,
                const double *mf_host, int nrhs, cudaStream_t st, const TileConfig *force,
                const int *gate = nullptr, int gate_stride = 0, const void *halo_up = nullptr,
                const void *halo_dn = nullptr, double *norm_partials = nullptr, int t_begin = 0,
-               int t_count = 0, const ResidualFuse *fuse = nullptr);
+               int t_count = 0, const ResidualFuse *fuse = nullptr, void *phi = nullptr);
+// Scratch of one call on `st`, from the lattice's pool (stream-ordered: allocated and
+// freed on the stream).  Null, and no error, where there is none to be had: on a
+// capturing stream, out of memory, or for a call that gains nothing from it.
+struct PhiScratch {
+  void *p = nullptr;
+  cudaStream_t st;
+  PhiScratch(dw_lattice *lat, int op, int prec, int nrhs, cudaStream_t st_);
+  ~PhiScratch() {
+    if (p) cudaFreeAsync(p, st);
+  }
+  PhiScratch(const PhiScratch &) = delete;
+  PhiScratch &operator=(const PhiScratch &) = delete;
+};
+// The FP64 D with its own phi pass (see phi_kernel): below 2^15 sites the extra launch
+// costs what the pass saves (192 of ~1100 operations per site: 10 us there).
+constexpr long long kPhiPassMinSites = 1 << 15;
 // CTAs per right-hand side of a stencil launch with tile `t` (the length of the
 // per-RHS rows of norm_partials).
 long long dslash_ctas_per_rhs(const dw_lattice *lat, TileConfig t);
@@ -105,8 +129,15 @@ int eo_merge(dw_lattice *lat, int prec, void *full, const void *even, const void
 // out = A in, A^-1 in, A^+ in or A^-+ in (A = alpha + beta K), on parity fields
 int apply_m5(dw_lattice *lat, int prec, void *out, const void *in, const double *mf, int nrhs,
              bool inv, bool dag, cudaStream_t st);
-// out (parity) = alpha own + beta K own + hscale Dhop (b + cK) nbr (OP_D), or the
-// D^+ form (OP_DDAG); own may be null
+// out = (1 + (c / b) K) A^-1 in (dag: the adjoint), on parity fields
+int apply_m5_inv_phi(dw_lattice *lat, int prec, void *out, const void *in, const double *mf,
+                     int nrhs, bool dag, cudaStream_t st, const int *gate, int gate_stride);
+// out = in + (c / b) K in = phi / b, on parity or whole-lattice fields
+int apply_phi(dw_lattice *lat, int prec, void *out, const void *in, bool parity_field,
+              const double *mf, int nrhs, cudaStream_t st, const int *gate, int gate_stride);
+// out (parity) = alpha own + beta K own + hscale Dhop (b + cK) nbr (OP_D; OP_HOP_LOCAL
+// with nbr already phi / b), or the D^+ form (OP_DDAG), or hscale b Dhop^+ nbr
+// (OP_HOP_SCALED_DAG); own may be null
 int run_dslash_cb(dw_lattice *lat, int prec, int op, void *out, const void *nbr, const void *own,
                   int parity, double alpha, double beta, double hscale, const double *mf,
                   int nrhs, cudaStream_t st, const int *gate, int gate_stride,

@@ -90,13 +90,17 @@ struct Solve {
   // One inner iteration over all RHS (masked by `run`).  <p, D^+D p> is
   // |D p|^2, summed per CTA by the D pass itself.
   int ctas_d() const {
-    return (int)(eo ? cb_ctas_per_rhs(lat, pp, OP_D)
+    return (int)(eo ? cb_ctas_per_rhs(lat, pp, OP_HOP_LOCAL)
                     : dslash_ctas_per_rhs(lat, pick_tile(lat, pp, OP_D, nrhs)));
   }
   int ctas_ddag() const {
     return (int)(eo ? cb_ctas_per_rhs(lat, pp, OP_DDAG)
                     : dslash_ctas_per_rhs(lat, pick_tile(lat, pp, OP_DDAG, nrhs)));
   }
+
+  // phi scratch of an FP64 D: a field that the D^+ pass behind it writes (or, with the
+  // fused update, leaves alone)
+  void *phi(void *field) const { return lat->V5 * nrhs >= kPhiPassMinSites ? field : nullptr; }
 
   // alpha follows from the D (Dhat) pass, |D p|^2, so the last launch of the
   // D^+ (Dhat^+) pass applies r_s -= alpha A p itself and leaves |r_s|^2 per CTA:
@@ -110,7 +114,7 @@ struct Solve {
                        kCGStateInts, w->dnorm);
     else
       rc = run_dslash(lat, pp, OP_D, w->tmp, w->p, mf, nrhs, st, nullptr, gate_run(),
-                      kCGStateInts, nullptr, nullptr, w->dnorm);
+                      kCGStateInts, nullptr, nullptr, w->dnorm, 0, 0, nullptr, phi(w->Ap));
     if (rc) return rc;
     if (cg_alpha(c, w->dnorm, nd, w->state, st))
       return cuda_fail(cudaGetLastError(), "cg iteration launch");
@@ -145,7 +149,7 @@ struct Solve {
                        gate_update(), kCGStateInts, nullptr);
     } else {
       rc = run_dslash(lat, DW_F64, OP_D, w->tmp64, x, mf, nrhs, st, nullptr, gate_update(),
-                      kCGStateInts);
+                      kCGStateInts, nullptr, nullptr, nullptr, 0, 0, nullptr, phi(w->Ax64));
       if (rc) return rc;
       rc = run_dslash(lat, DW_F64, OP_DDAG, w->Ax64, w->tmp64, mf, nrhs, st, nullptr,
                       gate_update(), kCGStateInts);
@@ -253,9 +257,11 @@ int cg_run(dw_lattice *lat, void *x, const void *b, const double *mf, int nrhs, 
   // tile choice for the inner operator of this solve (timed once per lattice
   // and RHS count, then cached; the FP64 operator of the reliable updates keeps
   // the untuned tile unless it is the inner operator)
-  for (int op : {(int)OP_D, (int)OP_DDAG}) {
-    if (eo)
+  for (int op : {(int)OP_D, (int)OP_DDAG, (int)OP_HOP_LOCAL}) {
+    if (eo && (S.pp != DW_F64 || op != OP_D))  // (the FP64 Dhat has no fused D hop)
       rc = tune_cb(lat, S.pp, op, st);
+    else if (eo || op > OP_DDAG)
+      continue;
     else if (!lat->tuned.count(std::make_tuple(S.pp, op, nrhs)))
       rc = tune_tile(lat, S.pp, op, nrhs, st, true);
     if (rc) return rc;
@@ -430,9 +436,9 @@ extern "C" int dw_solve_eo(dw_lattice *lat, void *x, const void *eta, const doub
       (rc = eo_split(lat, DW_F64, w->e1_64, w->xo, x, nrhs, st)))
     return rc;
   // bhat = eta_o - H_oe A^-1 eta_e
-  if ((rc = apply_m5(lat, DW_F64, w->e2_64, w->eta_e, mf, nrhs, true, false, st)) ||
-      (rc = run_dslash_cb(lat, DW_F64, OP_D, w->bhat, w->e2_64, w->eta_o, 1, 1.0, 0.0, 0.5, mf,
-                          nrhs, st, nullptr, 0, nullptr)))
+  if ((rc = apply_m5_inv_phi(lat, DW_F64, w->e2_64, w->eta_e, mf, nrhs, false, st, nullptr, 0)) ||
+      (rc = run_dslash_cb(lat, DW_F64, OP_HOP_LOCAL, w->bhat, w->e2_64, w->eta_o, 1, 1.0, 0.0, 0.5,
+                          mf, nrhs, st, nullptr, 0, nullptr)))
     return rc;
   // b' = Dhat^+ bhat, then CG on Dhat^+ Dhat x_o = b'
   if ((rc = apply_schur(lat, DW_F64, w->bpr, w->bhat, mf, nrhs, true, w->e1_64, w->e2_64, st,
@@ -456,11 +462,14 @@ extern "C" int dw_solve_eo(dw_lattice *lat, void *x, const void *eta, const doub
   // x_e = A^-1 (eta_e - H_eo x_o), x = (x_e, x_o), and |eta - D x|^2 per RHS in FP64
   auto reconstruct_and_residual = [&]() -> int {
     int r;
-    if ((r = run_dslash_cb(lat, DW_F64, OP_D, w->e1_64, w->xo, w->eta_e, 0, 1.0, 0.0, 0.5, mf,
-                           nrhs, st, nullptr, 0, nullptr)) ||
+    if ((r = apply_phi(lat, DW_F64, w->e2_64, w->xo, true, mf, nrhs, st, nullptr, 0)) ||
+        (r = run_dslash_cb(lat, DW_F64, OP_HOP_LOCAL, w->e1_64, w->e2_64, w->eta_e, 0, 1.0, 0.0,
+                           0.5, mf, nrhs, st, nullptr, 0, nullptr)) ||
         (r = apply_m5(lat, DW_F64, w->e2_64, w->e1_64, mf, nrhs, true, false, st)) ||
         (r = eo_merge(lat, DW_F64, x, w->e2_64, w->xo, nrhs, st)) ||
-        (r = run_dslash(lat, DW_F64, OP_D, w->Ax64, x, mf, nrhs, st, nullptr)))
+        (r = run_dslash(lat, DW_F64, OP_D, w->Ax64, x, mf, nrhs, st, nullptr, nullptr, 0, nullptr,
+                        nullptr, nullptr, 0, 0, nullptr,
+                        lat->V5 * nrhs >= kPhiPassMinSites ? w->r64 : nullptr)))
       return r;
     if (cg_residual(c, (double *)w->r64, (const double *)eta, (const double *)w->Ax64,
                     w->partials, nullptr, st) ||

@@ -196,7 +196,18 @@ __host__ __device__ __forceinline__ long long link_off(int x4, int mu, int nlv) 
 
 // ---------------------------------------------------------------------------
 // Operator kinds handled by the stencil kernel.
-enum OpKind { OP_DHOP = 0, OP_DHOP_DAG = 1, OP_D = 2, OP_DDAG = 3 };
+//   OP_HOP_LOCAL       D on an input that already is phi / b = psi + (c / b) K psi (one
+//                      streaming pass, phi_kernel in dw_eo.cu): local term of `own` plus
+//                      hscale * b * Dhop in
+//   OP_HOP_SCALED_DAG  hscale * b * Dhop^+ in, no local term
+enum OpKind {
+  OP_DHOP = 0,
+  OP_DHOP_DAG = 1,
+  OP_D = 2,
+  OP_DDAG = 3,
+  OP_HOP_LOCAL = 4,
+  OP_HOP_SCALED_DAG = 5
+};
 
 struct DslashParams {
   void *out;

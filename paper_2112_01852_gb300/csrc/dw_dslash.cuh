@@ -1162,8 +1162,9 @@ __device__ __forceinline__ void dslash_body(const DslashParams &p) {
   using C = typename P::C;
   using vec = typename P::vec;
   using V2 = typename Pair<P>::type;
-  constexpr bool DAG = (OP == OP_DHOP_DAG || OP == OP_DDAG);
+  constexpr bool DAG = (OP == OP_DHOP_DAG || OP == OP_DDAG || OP == OP_HOP_SCALED_DAG);
   constexpr bool PHI = (OP == OP_D);
+  constexpr bool LOCAL = (OP == OP_D || OP == OP_HOP_LOCAL);  // the D epilogue
   constexpr int SF = DAG ? 1 : -1;  // sign S of the forward hop
   constexpr int SB = -SF;           // sign S of the backward hop
 
@@ -1218,12 +1219,12 @@ __device__ __forceinline__ void dslash_body(const DslashParams &p) {
   vec *out = reinterpret_cast<vec *>(p.out) + (long long)rhs * p.rhs_stride;
   const vec *gauge = reinterpret_cast<const vec *>(p.gauge);
 
-  const C mf = (OP == OP_D || OP == OP_DDAG) ? (C)p.mf[rhs] : C(0);
+  const C mf = (LOCAL || OP == OP_DDAG) ? (C)p.mf[rhs] : C(0);
   // D's hop acts on phi / b = psi + (c / b) K psi: `c` is c / b for D, and the
   // factor b moves into the scale of the hop sum (hsc), so forming the
   // combination takes one FMA per element instead of an FMA and a multiply
   const C b = (C)p.b, c = PHI ? (C)(p.c / p.b) : (C)p.c;
-  const C hsc = PHI ? (C)(p.hscale * p.b) : (C)p.hscale;
+  const C hsc = (LOCAL || OP == OP_HOP_SCALED_DAG) ? (C)(p.hscale * p.b) : (C)p.hscale;
   const C alpha = (C)p.alpha, beta = (C)p.beta;
   // the field of the local term alpha psi + beta K psi (none: hopping term alone)
   Field<P> Fo;
@@ -1235,7 +1236,7 @@ __device__ __forceinline__ void dslash_body(const DslashParams &p) {
   SpinorP<P> acc[SPT];
   extern __shared__ __align__(16) unsigned char smem_raw[];
   size_t smem_used = 0;
-  double nsq = 0.0;     // OP_D: |out|^2 of this thread's output sites
+  double nsq = 0.0;     // LOCAL: |out|^2 of this thread's output sites
   bool stored = false;  // OP_D on the rows path: stored inside its loop
 
   int nb[8];   // neighbours in the order t+, t-, z+, z-, y+, y-, x+, x-
@@ -1511,7 +1512,21 @@ __device__ __forceinline__ void dslash_body(const DslashParams &p) {
 #pragma unroll
       for (int j = 0; j < SPT; ++j) store(j, acc[j]);
     }
-  } else if constexpr (OP == OP_D) {
+  } else if constexpr (OP == OP_HOP_SCALED_DAG) {
+    if (active) {
+#pragma unroll
+      for (int j = 0; j < SPT; ++j) {
+#pragma unroll
+        for (int cc = 0; cc < 3; ++cc) {
+          acc[j].up.re[cc] = p_mul(mhalf, acc[j].up.re[cc]);
+          acc[j].up.im[cc] = p_mul(mhalf, acc[j].up.im[cc]);
+          acc[j].lo.re[cc] = p_mul(mhalf, acc[j].lo.re[cc]);
+          acc[j].lo.im[cc] = p_mul(mhalf, acc[j].lo.im[cc]);
+        }
+        store(j, acc[j]);
+      }
+    }
+  } else if constexpr (LOCAL) {
     // out = alpha psi + beta K psi - 1/2 Dhop phi; optionally |out|^2 per CTA
     // (the CG's <p, D^+D p> = |D p|^2, fused here to save a pass over two fields)
     if (active && !stored)
@@ -1856,6 +1871,11 @@ int launch_variant(const DslashParams &p, int op, TileConfig cfg, cudaStream_t s
     case OP_DHOP_DAG: return launch_spt<P, OP_DHOP_DAG, VAR>(p, cfg, st);
     case OP_D: return launch_spt<P, OP_D, VAR>(p, cfg, st);
     case OP_DDAG: return launch_spt<P, OP_DDAG, VAR>(p, cfg, st);
+    case OP_HOP_LOCAL:  // FP64 register variant (see run_dslash)
+      if constexpr (std::is_same<typename P::C, double>::value && VAR == 0)
+        return launch_spt<P, OP_HOP_LOCAL, VAR>(p, cfg, st);
+      else
+        return -2;
   }
   return -2;
 }
@@ -1871,14 +1891,15 @@ int launch_variant_cplx(const DslashParams &p, int op, TileConfig cfg, cudaStrea
   return -2;
 }
 
-// Checkerboard entry points (the D and D^+ forms; Dhop is D with b = 1,
-// c = 0, no local term and factor 1).
+// Checkerboard entry points.
 template <class P, int VAR>
 int launch_variant_cb(const DslashParams &p, int op, TileConfig cfg, cudaStream_t st) {
   if (cfg.spt < 1 || p.Ls % cfg.spt) return -2;
   switch (op) {
     case OP_D: return launch_spt<P, OP_D, VAR, true>(p, cfg, st);
     case OP_DDAG: return launch_spt<P, OP_DDAG, VAR, true>(p, cfg, st);
+    case OP_HOP_LOCAL: return launch_spt<P, OP_HOP_LOCAL, VAR, true>(p, cfg, st);
+    case OP_HOP_SCALED_DAG: return launch_spt<P, OP_HOP_SCALED_DAG, VAR, true>(p, cfg, st);
   }
   return -2;
 }
@@ -1890,6 +1911,9 @@ int max_threads_variant(int op, int spt) {
     case OP_DHOP_DAG: return max_threads_op<P, OP_DHOP_DAG, VAR>(spt);
     case OP_D: return max_threads_op<P, OP_D, VAR>(spt);
     case OP_DDAG: return max_threads_op<P, OP_DDAG, VAR>(spt);
+    case OP_HOP_LOCAL:
+      if constexpr (std::is_same<typename P::C, double>::value && VAR == 0)
+        return max_threads_op<P, OP_HOP_LOCAL, VAR>(spt);
   }
   return 0;
 }

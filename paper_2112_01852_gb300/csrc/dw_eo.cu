@@ -36,8 +36,55 @@ struct M5Params {
   int nrhs;
   int dag;
   double alpha, beta;
+  double cb;  // c / b of the (b + cK) factor fused behind A^-1
+  const int *gate;  // optional: RHS r runs only if gate[r * gate_stride] != 0
+  int gate_stride;
   double mf[kMaxRhsPerLaunch];
 };
+
+// out = psi + (c / b) K psi (phi / b) over whole-lattice or parity fields, one thread
+// per (site, half, colour) walking s; the rounding is that of roll_5d's unit form, so
+// a hop of its output equals the fused D bit for bit.  Bound by HBM (two field
+// accesses).  At FP64 the fused D rebuilds phi at each of a site's eight neighbours:
+// 192 of its ~1100 FP64 operations per site, on the pipe that bounds it; this pass
+// does it once.
+template <class P>
+__global__ void phi_kernel(const M5Params q) {
+  using C = typename P::C;
+  using vec = typename P::vec;
+  using V2 = typename Pair<P>::type;
+  constexpr int NPV = 24 / P::R;
+  constexpr int VPQ = 4 / P::R;
+  const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long per_rhs = q.nsite * 6;
+  if (gid >= per_rhs * q.nrhs) return;
+  const int rhs = (int)(gid / per_rhs);
+  if (q.gate && !q.gate[(long long)rhs * q.gate_stride]) return;
+  const long long rem = gid - (long long)rhs * per_rhs;
+  const int comp = (int)(rem / q.nsite);  // half * 3 + colour
+  const int site = (int)(rem - (long long)comp * q.nsite);
+  const int Ls = q.Ls;
+  const vec *in = reinterpret_cast<const vec *>(q.in) + (long long)rhs * q.rhs_stride;
+  vec *out = reinterpret_cast<vec *>(q.out) + (long long)rhs * q.rhs_stride;
+  const long long off = (long long)comp * VPQ * kPlaneStride;
+  // the upper spins take slice s-1, the lower ones s+1: walk s down or up so that the
+  // neighbour is the next element read
+  const bool lower = comp >= 3;
+  auto at = [&](int k) { return site_off(site, lower ? k : Ls - 1 - k, Ls, NPV) + off; };
+  const C c = (C)q.cb, mf = (C)q.mf[rhs];
+  V2 fr, fi, cr, ci;
+  quad_in_h<HINT_NONE>(fr, fi, in + at(0), kPlaneStride, 0ull);
+  cr = fr;
+  ci = fi;
+  for (int k = 0; k < Ls; ++k) {
+    V2 nr = fr, ni = fi;  // the element that follows the wall is the first one, with -mf
+    if (k + 1 < Ls) quad_in_h<HINT_NONE>(nr, ni, in + at(k + 1), kPlaneStride, 0ull);
+    const V2 w = bc<V2>(k + 1 < Ls ? c : c * -mf);
+    quad_out(out + at(k), kPlaneStride, p_fma(w, nr, cr), p_fma(w, ni, ci));
+    cr = nr;
+    ci = ni;
+  }
+}
 
 // A = alpha + beta K along s for one (site, half, colour).  In the forward
 // orientation the half couples slice s to s-1 and slice 0 to Ls-1 with -mf:
@@ -46,7 +93,10 @@ struct M5Params {
 // two are the same on the reversed slice order.  The inverse solves it with
 // y_0 = (x_0 + mf g sum_{k=1}^{Ls-1} (-g)^{Ls-1-k} x_k) / (alpha (1 + mf (-g)^Ls)),
 // g = beta / alpha, then y_s = (x_s - beta y_{s-1}) / alpha.
-template <class P, bool INV>
+// PHI (inverse only): out = (1 + (c / b) K) A^-1 in, or its adjoint (polynomials of
+// one K commute, so both orders are the same): the (b + cK) of the hop that reads the
+// output, or of the adjoint hop that wrote the input, costs no pass of its own.
+template <class P, bool INV, bool PHI = false>
 __global__ void m5_kernel(const M5Params q) {
   using C = typename P::C;
   using vec = typename P::vec;
@@ -57,6 +107,7 @@ __global__ void m5_kernel(const M5Params q) {
   const long long per_rhs = q.nsite * 6;
   if (gid >= per_rhs * q.nrhs) return;
   const int rhs = (int)(gid / per_rhs);
+  if (q.gate && !q.gate[(long long)rhs * q.gate_stride]) return;
   long long rem = gid - (long long)rhs * per_rhs;
   const int comp = (int)(rem / q.nsite);  // half * 3 + colour
   const int site = (int)(rem - (long long)comp * q.nsite);
@@ -104,14 +155,23 @@ __global__ void m5_kernel(const M5Params q) {
     V2 x0r, x0i;
     ld(0, x0r, x0i);
     V2 yr = p_mul(den, p_fma(mfg, hr, x0r)), yi = p_mul(den, p_fma(mfg, hi, x0i));
-    quad_out(out + at(0), kPlaneStride, yr, yi);
+    const V2 y0r = yr, y0i = yi, cb = bc<V2>((C)q.cb);
+    if (!PHI) quad_out(out + at(0), kPlaneStride, yr, yi);
     const V2 ra = bc<V2>(C(1) / al), mb = bc<V2>(-be);
     for (int k = 1; k < Ls; ++k) {
       V2 xr, xi;
       ld(k, xr, xi);
+      const V2 pr_ = yr, pi_ = yi;
       yr = p_mul(ra, p_fma(mb, yr, xr));
       yi = p_mul(ra, p_fma(mb, yi, xi));
-      quad_out(out + at(k), kPlaneStride, yr, yi);
+      if (PHI)
+        quad_out(out + at(k), kPlaneStride, p_fma(cb, pr_, yr), p_fma(cb, pi_, yi));
+      else
+        quad_out(out + at(k), kPlaneStride, yr, yi);
+    }
+    if (PHI) {  // slice 0 takes the last one with -mf
+      const V2 w = bc<V2>((C)q.cb * -mf);
+      quad_out(out + at(0), kPlaneStride, p_fma(w, yr, y0r), p_fma(w, yi, y0i));
     }
   }
 }
@@ -186,20 +246,57 @@ int launch_split(dw_lattice *lat, int prec, void *full, void *even, void *odd, i
   return e == cudaSuccess ? DW_OK : cuda_fail(e, "split launch");
 }
 
+enum M5Kind { M5_A, M5_INV, M5_INV_PHI, M5_PHI };
+
 template <class P>
-int launch_m5_p(const M5Params &q, bool inv, cudaStream_t st) {
+int launch_m5_p(const M5Params &q, M5Kind kind, cudaStream_t st) {
   const long long n = q.nsite * 6 * q.nrhs;
   const unsigned blocks = (unsigned)((n + 255) / 256);
-  if (inv)
-    m5_kernel<P, true><<<blocks, 256, 0, st>>>(q);
-  else
-    m5_kernel<P, false><<<blocks, 256, 0, st>>>(q);
+  switch (kind) {
+    case M5_A: m5_kernel<P, false><<<blocks, 256, 0, st>>>(q); break;
+    case M5_INV: m5_kernel<P, true><<<blocks, 256, 0, st>>>(q); break;
+    case M5_INV_PHI: m5_kernel<P, true, true><<<blocks, 256, 0, st>>>(q); break;
+    case M5_PHI: phi_kernel<P><<<blocks, 256, 0, st>>>(q); break;
+  }
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? DW_OK : cuda_fail(e, "m5 launch");
 }
 
+// One fifth-dimension pass over nrhs fields of nsite sites (whole-lattice or parity).
+int run_m5(dw_lattice *lat, int prec, void *out, const void *in, long long nsite,
+           const double *mf, int nrhs, M5Kind kind, bool dag, const int *gate, int gate_stride,
+           cudaStream_t st) {
+  const size_t rb = (size_t)24 * (size_t)padded_v4(nsite) * lat->Ls * prec_real_bytes(prec);
+  for (int r0 = 0; r0 < nrhs; r0 += kMaxRhsPerLaunch) {
+    const int n = (nrhs - r0) < kMaxRhsPerLaunch ? (nrhs - r0) : kMaxRhsPerLaunch;
+    M5Params q;
+    memset(&q, 0, sizeof(q));
+    q.out = (char *)out + (size_t)r0 * rb;
+    q.in = (const char *)in + (size_t)r0 * rb;
+    q.nsite = nsite;
+    q.rhs_stride = padded_v4(nsite) * lat->Ls * (24 / prec_reals_per_vec(prec));
+    q.Ls = lat->Ls;
+    q.nrhs = n;
+    q.dag = dag ? 1 : 0;
+    q.alpha = lat->b * (4.0 - lat->M5) + 1.0;
+    q.beta = lat->c * (4.0 - lat->M5) - 1.0;
+    q.cb = lat->c / lat->b;
+    q.gate = gate ? gate + (size_t)r0 * gate_stride : nullptr;
+    q.gate_stride = gate_stride;
+    for (int r = 0; r < n; ++r) q.mf[r] = mf[r0 + r];
+    int rc;
+    switch (prec) {
+      case DW_F64: rc = launch_m5_p<F64>(q, kind, st); break;
+      case DW_F32: rc = launch_m5_p<F32>(q, kind, st); break;
+      default: rc = launch_m5_p<F16>(q, kind, st); break;
+    }
+    if (rc) return rc;
+  }
+  return DW_OK;
+}
+
 // Tile of the checkerboard stencil: two slices per thread where Ls allows,
-// 32-site tiles, the register variant (capped at FP32 / FP16), and for D at
+// 32-site tiles, the register variant (capped at FP32 / FP16), and but for D^+ at
 // FP32 / FP16 the slice groups split over three (else two) CTAs, as the tuner
 // prefers on the full lattice (D^+ keeps all slices in one CTA).
 // Key of a tuned checkerboard tile in the lattice's tile map (its own op codes).
@@ -213,7 +310,7 @@ TileConfig cb_default_tile(const dw_lattice *lat, int prec, int op) {
   t.zblk = auto_zblk(lat, prec);
   const int nchunk = lat->Ls / t.spt;
   t.sgrp = 1;
-  if (op == OP_D && prec != DW_F64)
+  if (op != OP_DDAG && prec != DW_F64)
     for (int g : {3, 2})
       if (nchunk % g == 0) {
         t.sgrp = g;
@@ -223,6 +320,7 @@ TileConfig cb_default_tile(const dw_lattice *lat, int prec, int op) {
 }
 
 TileConfig cb_tile(const dw_lattice *lat, int prec, int op) {
+  if (op == OP_HOP_SCALED_DAG) op = OP_HOP_LOCAL;  // the same hop: one tuned tile
   auto it = lat->tuned.find(std::make_tuple(prec, kCbOpKey + op, 0));
   return it != lat->tuned.end() ? it->second : cb_default_tile(lat, prec, op);
 }
@@ -254,31 +352,20 @@ int eo_merge(dw_lattice *lat, int prec, void *full, const void *even, const void
 
 int apply_m5(dw_lattice *lat, int prec, void *out, const void *in, const double *mf, int nrhs,
              bool inv, bool dag, cudaStream_t st) {
-  const long long nsite = lat->V4 / 2;
-  for (int r0 = 0; r0 < nrhs; r0 += kMaxRhsPerLaunch) {
-    const int n = (nrhs - r0) < kMaxRhsPerLaunch ? (nrhs - r0) : kMaxRhsPerLaunch;
-    M5Params q;
-    memset(&q, 0, sizeof(q));
-    const size_t rb = cb_field_bytes(lat, prec, 1);
-    q.out = (char *)out + (size_t)r0 * rb;
-    q.in = (const char *)in + (size_t)r0 * rb;
-    q.nsite = nsite;
-    q.rhs_stride = padded_v4(nsite) * lat->Ls * (24 / prec_reals_per_vec(prec));
-    q.Ls = lat->Ls;
-    q.nrhs = n;
-    q.dag = dag ? 1 : 0;
-    q.alpha = lat->b * (4.0 - lat->M5) + 1.0;
-    q.beta = lat->c * (4.0 - lat->M5) - 1.0;
-    for (int r = 0; r < n; ++r) q.mf[r] = mf[r0 + r];
-    int rc;
-    switch (prec) {
-      case DW_F64: rc = launch_m5_p<F64>(q, inv, st); break;
-      case DW_F32: rc = launch_m5_p<F32>(q, inv, st); break;
-      default: rc = launch_m5_p<F16>(q, inv, st); break;
-    }
-    if (rc) return rc;
-  }
-  return DW_OK;
+  return run_m5(lat, prec, out, in, lat->V4 / 2, mf, nrhs, inv ? M5_INV : M5_A, dag, nullptr, 0,
+                st);
+}
+
+int apply_m5_inv_phi(dw_lattice *lat, int prec, void *out, const void *in, const double *mf,
+                     int nrhs, bool dag, cudaStream_t st, const int *gate, int gate_stride) {
+  return run_m5(lat, prec, out, in, lat->V4 / 2, mf, nrhs, M5_INV_PHI, dag, gate, gate_stride,
+                st);
+}
+
+int apply_phi(dw_lattice *lat, int prec, void *out, const void *in, bool parity_field,
+              const double *mf, int nrhs, cudaStream_t st, const int *gate, int gate_stride) {
+  return run_m5(lat, prec, out, in, parity_field ? lat->V4 / 2 : lat->V4, mf, nrhs, M5_PHI, false,
+                gate, gate_stride, st);
 }
 
 long long cb_ctas_per_rhs(const dw_lattice *lat, int prec, int op) {
@@ -350,22 +437,40 @@ int run_dslash_cb(dw_lattice *lat, int prec, int op, void *out, const void *nbr,
 // out_o = Dhat in_o (dag: Dhat^+ in_o) at precision prec; t1, t2: even-parity
 // scratch fields; norm_partials (optional, not dag) receives |out|^2 per CTA;
 // fuse (optional, dag only): the CG residual update in place of storing out.
+// The (b + cK) of the second hop of Dhat and of the first of Dhat^+ rides in the
+// A^-1 pass, so those two are the plain hopping term: no phi per neighbour, no slice
+// exchange (24^4 x 16 FP32: Dhat and Dhat^+ together 1.09 -> 1.01 ms).
 int apply_schur(dw_lattice *lat, int prec, void *out, const void *in, const double *mf, int nrhs,
                 bool dag, void *t1, void *t2, cudaStream_t st, const int *gate, int gate_stride,
                 double *norm_partials, const ResidualFuse *fuse) {
-  const int op = dag ? OP_DDAG : OP_D;
   const double alpha = lat->b * (4.0 - lat->M5) + 1.0;
   const double beta = lat->c * (4.0 - lat->M5) - 1.0;
-  // t1 = H_eo in   (dag: H_oe^+ in), on even sites
-  int rc = run_dslash_cb(lat, prec, op, t1, in, nullptr, 0, 0.0, 0.0, -0.5, mf, nrhs, st, gate,
-                         gate_stride, nullptr);
-  if (rc) return rc;
-  // t2 = A^-1 t1   (A^-+)
-  if ((rc = apply_m5(lat, prec, t2, t1, mf, nrhs, true, dag, st))) return rc;
-  // out = A in - H_oe t2  (A^+ in - H_eo^+ t2), on odd sites
-  return run_dslash_cb(lat, prec, op, out, t2, in, 1, alpha, beta, 0.5, mf, nrhs, st, gate,
-                       gate_stride, dag ? nullptr : norm_partials, nullptr,
-                       dag ? fuse : nullptr);
+  int rc;
+  if (dag) {
+    // t1 = -b/2 Dhop^+ in on even sites, t2 = (1 + (c/b) K^+) A^-+ t1
+    if ((rc = run_dslash_cb(lat, prec, OP_HOP_SCALED_DAG, t1, in, nullptr, 0, 0.0, 0.0, -0.5, mf,
+                            nrhs, st, gate, gate_stride, nullptr)) ||
+        (rc = apply_m5_inv_phi(lat, prec, t2, t1, mf, nrhs, true, st, gate, gate_stride)))
+      return rc;
+    // out = A^+ in - H_eo^+ t2 on odd sites
+    return run_dslash_cb(lat, prec, OP_DDAG, out, t2, in, 1, alpha, beta, 0.5, mf, nrhs, st, gate,
+                         gate_stride, nullptr, nullptr, fuse);
+  }
+  // t1 = H_eo in on even sites
+  if (prec == DW_F64) {  // phi in its own pass (see phi_kernel); out is free until the end
+    if ((rc = apply_phi(lat, prec, out, in, true, mf, nrhs, st, gate, gate_stride)) ||
+        (rc = run_dslash_cb(lat, prec, OP_HOP_LOCAL, t1, out, nullptr, 0, 0.0, 0.0, -0.5, mf, nrhs,
+                            st, gate, gate_stride, nullptr)))
+      return rc;
+  } else if ((rc = run_dslash_cb(lat, prec, OP_D, t1, in, nullptr, 0, 0.0, 0.0, -0.5, mf, nrhs, st,
+                                 gate, gate_stride, nullptr))) {
+    return rc;
+  }
+  // t2 = (1 + (c/b) K) A^-1 t1, out = A in - H_oe A^-1 t1 on odd sites
+  if ((rc = apply_m5_inv_phi(lat, prec, t2, t1, mf, nrhs, false, st, gate, gate_stride)))
+    return rc;
+  return run_dslash_cb(lat, prec, OP_HOP_LOCAL, out, t2, in, 1, alpha, beta, 0.5, mf, nrhs, st,
+                       gate, gate_stride, norm_partials);
 }
 
 // Times the checkerboard tiles of (prec, op) on two scratch parity fields (the
@@ -402,7 +507,7 @@ int tune_cb(dw_lattice *lat, int prec, int op, cudaStream_t st) {
           cudaGetLastError();
           continue;  // not launchable (CTA limits)
         }
-        float ms[3];
+        float ms[2];
         for (float &m : ms) {
           cudaEventRecord(e0, st);
           run_dslash_cb(lat, prec, op, lat->stage_out, lat->stage_in, nullptr, 0, 0.0, 0.0, -0.5,
@@ -412,9 +517,8 @@ int tune_cb(dw_lattice *lat, int prec, int op, cudaStream_t st) {
           m = 1e30f;
           if (cudaEventElapsedTime(&m, e0, e1) != cudaSuccess) m = 1e30f;
         }
-        std::sort(ms, ms + 3);
-        if (ms[1] < best) {
-          best = ms[1];
+        if (std::min(ms[0], ms[1]) < best) {
+          best = std::min(ms[0], ms[1]);
           best_t = t;
         }
       }

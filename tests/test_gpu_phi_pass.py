@@ -1,0 +1,45 @@
+"""The FP64 D with its (b + cK) pass: bit for bit the fused kernel, which a capturing
+stream takes (no allocation there), and within the oracle's tolerance."""
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+import oracle  # noqa: E402
+from gpu_helpers import TOL, make_case  # noqa: E402
+from paper_2112_01852_gb300 import dw  # noqa: E402
+from paper_2112_01852_gb300.lattice import Lattice  # noqa: E402
+
+
+# V5 nrhs just below and at the 2^15 threshold of the pass, ragged extents, odd Ls, Ls = 1
+@pytest.mark.parametrize("dims,Ls,nrhs,kind", [
+    ((8, 8, 8, 8), 8, 1, dw.DW_MOBIUS), ((7, 9, 5, 11), 9, 2, dw.DW_MOBIUS),
+    ((8, 8, 8, 8), 7, 1, dw.DW_MOBIUS), ((16, 16, 8, 16), 1, 1, dw.DW_MOBIUS),
+    ((8, 4, 8, 16), 8, 3, dw.DW_SHAMIR)])
+def test_phi_pass_equals_fused(dims, Ls, nrhs, kind):
+    U, psi = make_case(dims, Ls, nrhs, 11)
+    mfs = [0.01 + 0.02 * r for r in range(nrhs)]
+    lat = Lattice(dims, Ls, kind=kind, prec=dw.DW_F64)
+    lat.load_gauge(U)
+    x = lat.pack(psi)
+    y, ref = lat.empty(nrhs), lat.empty(nrhs)
+    y.zero_()
+    ref.zero_()
+    lat.D(ref, x, mfs, nrhs)  # loads the kernels before the capture
+    lat.D(y, x, mfs, nrhs)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        lat.D(ref, x, mfs, nrhs)
+    ref.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(y, ref)
+    got = lat.unpack(y, nrhs)
+    b, c = (1.5, 0.5) if kind == dw.DW_MOBIUS else (1.0, 0.0)
+    want = np.concatenate([oracle.dw(psi[r:r + 1], U, dims, Ls, 1.8, b, c, mfs[r])
+                           for r in range(nrhs)])
+    assert oracle.rel_l2(got, want) <= TOL[dw.DW_F64]
+    lat.close()
