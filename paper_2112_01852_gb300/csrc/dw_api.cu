@@ -108,10 +108,49 @@ int auto_zblk(const dw_lattice *lat, int prec) {
   return lat->dims[2];
 }
 
-// Untuned choice: the smallest slices-per-thread whose CTA of 32 sites x Ls/spt
-// slice groups fits the kernel's register budget, then up to 256 threads.
+static int largest_divisor(int n, int cap) {
+  for (int d = cap < n ? cap : n; d > 1; --d)
+    if (n % d == 0) return d;
+  return 1;
+}
+
+// Untuned register tile at FP32 / FP16: the capped variant, two slices per thread (three
+// or one at an odd Ls) share a link, and CTAs of 32 sites by two slice groups (D^+: all of
+// them up to eight, its slices being combined in the CTA) keep 16 warps on an SM.  Within
+// 12 % (FP16 15 %) of the best of all tiles over 12^3 x 24 x 10 .. 32^3 x 64 x 12, where one
+// thread row per slice and variant 0 took 1.3 - 2.2 times the best.
+TileConfig register_tile(const dw_lattice *lat, int prec, int op, int nrhs) {
+  const int Ls = lat->Ls;
+  if (prec != DW_F64 && !(lat->cplx && prec == DW_F32)) {
+    const int spt = Ls % 2 == 0 ? 2 : (Ls % 3 == 0 ? 3 : 1);
+    const int nchunk = Ls / spt, cpc = largest_divisor(nchunk, op == OP_DDAG ? 8 : 2);
+    // several RHS: one sweep after another (see dw_tune), each with its own reuse window
+    const TileConfig t{spt, 32, 4, auto_zblk(lat, prec), nchunk / cpc, nrhs > 1 ? 1 : 0};
+    if (tile_valid(lat, prec, op, t)) return t;
+  }
+  return generic_tile(lat, prec, op);
+}
+
+// Untuned choice.  The hopping terms stage their tile's rows in shared memory (variant 6)
+// where the planes allow it: Dhop with two slices per CTA and the widest tile of 128, 96,
+// 64 or 32 sites (at most 8 % from the best tile), D the same way at FP16 (64 sites by
+// two slice groups) and in planes of 96-site tiles; elsewhere D's register tile is as good.
 TileConfig default_tile(const dw_lattice *lat, int prec, int op, int nrhs) {
-  (void)nrhs;
+  TileConfig t = register_tile(lat, prec, op, nrhs);
+  if (t.variant != 4 || t.spt != 2 || op == OP_DDAG) return t;
+  const int nblk = lat->dims[0] * lat->dims[1] / 32, nchunk = lat->Ls / 2;
+  const bool three = nblk % 3 == 0 && nblk % 4 != 0;
+  if (op == OP_D && prec == DW_F32 && !three) return t;
+  t.variant = 6;
+  t.tx = op == OP_D && prec == DW_F16 ? 64 : (three ? 96 : 128);
+  while (t.tx > 32 && (t.tx % 96 == 0 ? nblk % 3 : nblk % (t.tx / 32))) t.tx = t.tx == 96 ? 64 : t.tx / 2;
+  t.sgrp = nchunk / largest_divisor(nchunk, op == OP_D ? 2 : (t.tx < 96 ? 2 : 1));
+  return tile_valid(lat, prec, op, t) ? t : register_tile(lat, prec, op, nrhs);
+}
+
+// The smallest slices-per-thread whose CTA of 32 sites x Ls/spt slice groups fits the
+// kernel's register budget, then up to 256 threads.
+TileConfig generic_tile(const dw_lattice *lat, int prec, int op) {
   const int Ls = lat->Ls;
   TileConfig t{0, 32, 0, auto_zblk(lat, prec), 1};
   // interleaved-complex FP32 fields: the capped register variant
@@ -647,7 +686,8 @@ int dw_apply_op_halo(dw_lattice *lat, int op, void *out, const void *in, const v
   if (!recv_up || !recv_dn) return fail(DW_ERR_ARG, "halo pointer is NULL");
   if (!aligned16(recv_up) || !aligned16(recv_dn))
     return fail(DW_ERR_ARG, "halos must be 16-byte aligned");
-  TileConfig t = default_tile(lat, lat->prec, op, nrhs);  // the halo path is variant 0
+  // the register variants take the faces (those that stage rows do not)
+  const TileConfig t = register_tile(lat, lat->prec, op, nrhs);
   return run_dslash(lat, lat->prec, op, out, in, op >= DW_OP_D ? mf : nullptr, nrhs,
                     (cudaStream_t)stream, &t, nullptr, 0, recv_up, recv_dn);
 }

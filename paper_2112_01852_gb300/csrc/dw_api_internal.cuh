@@ -64,6 +64,8 @@ size_t field_bytes(const dw_lattice *lat, int prec, int nrhs);
 FieldGeom geom(const dw_lattice *lat);
 int ensure_buffer(void **buf, size_t *cap, size_t need);
 TileConfig default_tile(const dw_lattice *lat, int prec, int op, int nrhs);
+TileConfig register_tile(const dw_lattice *lat, int prec, int op, int nrhs);
+TileConfig generic_tile(const dw_lattice *lat, int prec, int op);
 int auto_zblk(const dw_lattice *lat, int prec);
 TileConfig pick_tile(dw_lattice *lat, int prec, int op, int nrhs);
 bool tile_valid(const dw_lattice *lat, int prec, int op, TileConfig t);

@@ -20,6 +20,7 @@
 #pragma once
 
 #include <cooperative_groups.h>
+#include <atomic>
 #include <type_traits>
 
 #include "dw_common.cuh"
@@ -1841,18 +1842,29 @@ int launch_spt(const DslashParams &p, TileConfig cfg, cudaStream_t st) {
   }
 }
 
+// (queried once per kernel: the tile rules ask on every call)
+template <class P, int OP, int SPT, int VAR>
+int kernel_max_threads() {
+  static std::atomic<int> n{0};
+  int v = n.load(std::memory_order_relaxed);
+  if (!v) {
+    cudaFuncAttributes fa;
+    if (cudaFuncGetAttributes(&fa, dslash_entry<P, OP, SPT, VAR>()) != cudaSuccess) return 0;
+    v = fa.maxThreadsPerBlock;
+    n.store(v, std::memory_order_relaxed);
+  }
+  return v;
+}
+
 template <class P, int OP, int VAR>
 int max_threads_var(int spt) {
-  cudaFuncAttributes fa;
-  cudaError_t e;
   switch (spt) {
-    case 1: e = cudaFuncGetAttributes(&fa, dslash_entry<P, OP, 1, VAR>()); break;
-    case 2: e = cudaFuncGetAttributes(&fa, dslash_entry<P, OP, 2, VAR>()); break;
-    case 3: e = cudaFuncGetAttributes(&fa, dslash_entry<P, OP, 3, VAR>()); break;
-    case 4: e = cudaFuncGetAttributes(&fa, dslash_entry<P, OP, 4, VAR>()); break;
-    default: return 0;
+    case 1: return kernel_max_threads<P, OP, 1, VAR>();
+    case 2: return kernel_max_threads<P, OP, 2, VAR>();
+    case 3: return kernel_max_threads<P, OP, 3, VAR>();
+    case 4: return kernel_max_threads<P, OP, 4, VAR>();
   }
-  return e == cudaSuccess ? fa.maxThreadsPerBlock : 0;
+  return 0;
 }
 
 // Largest CTA that (op, spt) of variant VAR can launch: register limit and, for
