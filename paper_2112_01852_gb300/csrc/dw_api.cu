@@ -114,38 +114,68 @@ static int largest_divisor(int n, int cap) {
   return 1;
 }
 
-// Untuned register tile at FP32 / FP16: the capped variant, two slices per thread (three
-// or one at an odd Ls) share a link, and CTAs of 32 sites by two slice groups (D^+: all of
-// them up to eight, its slices being combined in the CTA) keep 16 warps on an SM.  Within
-// 12 % (FP16 15 %) of the best of all tiles over 12^3 x 24 x 10 .. 32^3 x 64 x 12, where one
-// thread row per slice and variant 0 took 1.3 - 2.2 times the best.
+// Untuned register tile (the variants that take t faces: 0 and 4), 32 sites wide.
+//  FP32 / FP16: the capped variant; two slices per thread share a link (D^+ at an odd Ls
+//  three, else one), one where the lattice would not fill the SMs with 8 warps each; CTAs of
+//  two slice groups (three at an odd Ls) keep 16 warps on an SM, D^+ up to eight groups, its
+//  slices being combined in the CTA.
+//  FP64: one slice per thread (D^+ two) and at most four groups per CTA: the kernels are
+//  bound by the FP64 pipe, and small CTAs balance it over the SMs (16^4 x 16 D 1.90 -> 1.78,
+//  D^+ 1.86 -> 1.76 ms; 10 x 12 x 8 x 20 x 10 D 0.53 -> 0.42).
+// With default_tile's choices within 8 % (FP16 15 %) of the best of all tiles on most of
+// 9^3 x 10 x 5 .. 32^3 x 64 x 12, where one thread row per slice and variant 0 took 1.1 - 2.2
+// times the best.
 TileConfig register_tile(const dw_lattice *lat, int prec, int op, int nrhs) {
   const int Ls = lat->Ls;
-  if (prec != DW_F64 && !(lat->cplx && prec == DW_F32)) {
-    const int spt = Ls % 2 == 0 ? 2 : (Ls % 3 == 0 ? 3 : 1);
-    const int nchunk = Ls / spt, cpc = largest_divisor(nchunk, op == OP_DDAG ? 8 : 2);
-    // several RHS: one sweep after another (see dw_tune), each with its own reuse window
-    const TileConfig t{spt, 32, 4, auto_zblk(lat, prec), nchunk / cpc, nrhs > 1 ? 1 : 0};
-    if (tile_valid(lat, prec, op, t)) return t;
-  }
-  return generic_tile(lat, prec, op);
+  if (lat->cplx && prec == DW_F32) return generic_tile(lat, prec, op);
+  const bool f64 = prec == DW_F64, even = Ls % 2 == 0;
+  int spt = even ? 2 : (op == OP_DDAG && Ls % 3 == 0 ? 3 : 1);
+  if (f64 ? op != OP_DDAG : even && lat->V5 * nrhs <= 64LL * 8 * lat->num_sms) spt = 1;
+  const int nchunk = Ls / spt;
+  int cpc = largest_divisor(nchunk, f64 ? 4 : (op == OP_DDAG ? 8 : (even ? 2 : 3)));
+  if (cpc == 1 && f64) cpc = largest_divisor(nchunk, 8);  // a prime Ls
+  // several RHS: one sweep after another (see dw_tune), each with its own reuse window
+  const TileConfig t{spt,  32, f64 ? 0 : 4, auto_zblk(lat, prec), nchunk / cpc,
+                     nrhs > 1 && !f64 ? 1 : 0};
+  return tile_valid(lat, prec, op, t) ? t : generic_tile(lat, prec, op);
 }
 
-// Untuned choice.  The hopping terms stage their tile's rows in shared memory (variant 6)
-// where the planes allow it: Dhop with two slices per CTA and the widest tile of 128, 96,
-// 64 or 32 sites (at most 8 % from the best tile), D the same way at FP16 (64 sites by
-// two slice groups) and in planes of 96-site tiles; elsewhere D's register tile is as good.
+// Untuned choice: the register tile, or where it was faster
+//  - Dhop at FP32 / FP16 (and D at FP16): the rows of a tile staged in shared memory
+//    (variant 6) where planes and Ls allow tiles of 64 sites or more, Dhop with two slices
+//    per CTA and the widest tile of 128, 96 and 64 sites, D with 64 sites and two groups;
+//  - D at FP32, and at an odd multiple of three slices: three or four slices per thread
+//    uncapped (variant 3: its loads of the s-neighbours shared by more slices);
+//  - an odd Ls at FP16: the prefetch variant 3;
+//  - Dhop at FP64: the prefetch variant 2 (16^4 x 16 1.65 -> 1.53 ms).
+// All of them sum the hops in the same order: the choice does not change a result.
 TileConfig default_tile(const dw_lattice *lat, int prec, int op, int nrhs) {
-  TileConfig t = register_tile(lat, prec, op, nrhs);
-  if (t.variant != 4 || t.spt != 2 || op == OP_DDAG) return t;
-  const int nblk = lat->dims[0] * lat->dims[1] / 32, nchunk = lat->Ls / 2;
-  const bool three = nblk % 3 == 0 && nblk % 4 != 0;
-  if (op == OP_D && prec == DW_F32 && !three) return t;
-  t.variant = 6;
-  t.tx = op == OP_D && prec == DW_F16 ? 64 : (three ? 96 : 128);
-  while (t.tx > 32 && (t.tx % 96 == 0 ? nblk % 3 : nblk % (t.tx / 32))) t.tx = t.tx == 96 ? 64 : t.tx / 2;
-  t.sgrp = nchunk / largest_divisor(nchunk, op == OP_D ? 2 : (t.tx < 96 ? 2 : 1));
-  return tile_valid(lat, prec, op, t) ? t : register_tile(lat, prec, op, nrhs);
+  const TileConfig base = register_tile(lat, prec, op, nrhs);
+  const int Ls = lat->Ls;
+  TileConfig t = base;
+  if (lat->cplx && prec == DW_F32) return base;
+  if (prec == DW_F64) {
+    if (op == OP_DDAG || op == OP_D || base.variant != 0) return base;
+    t.variant = 2;
+    return tile_valid(lat, prec, op, t) ? t : base;
+  }
+  if (base.variant != 4 || (Ls % 2 == 0 && base.spt == 1)) return base;
+  const int plane = lat->dims[0] * lat->dims[1], nblk = plane / 32;
+  const int blocks = (plane + 31) / 32;  // 32-site tiles of a plane
+  if (op == OP_D && (prec == DW_F32 || Ls % 2) && (Ls % 3 == 0 || Ls % 4 == 0)) {
+    t.variant = 3;
+    t.spt = Ls % 3 == 0 ? 3 : 4;
+    t.tx = Ls % 2 == 0 && (blocks % 2 == 0 || blocks >= 20) ? 64 : 32;
+    t.sgrp = (Ls / t.spt) / largest_divisor(Ls / t.spt, Ls % 2 == 0 ? 2 : 1);
+  } else if (Ls % 2) {
+    if (prec == DW_F32 || (op == OP_DDAG && Ls % 3 == 0)) return base;
+    t.variant = 3;
+  } else if (op != OP_DDAG && !(op == OP_D && prec == DW_F32) && plane % 32 == 0) {
+    t.variant = 6;
+    t.tx = op == OP_D ? 64 : (nblk % 4 == 0 ? 128 : (nblk % 3 == 0 ? 96 : 64));
+    t.sgrp = (Ls / 2) / largest_divisor(Ls / 2, op == OP_D || t.tx == 64 ? 2 : 1);
+  }
+  return tile_valid(lat, prec, op, t) ? t : base;
 }
 
 // The smallest slices-per-thread whose CTA of 32 sites x Ls/spt slice groups fits the

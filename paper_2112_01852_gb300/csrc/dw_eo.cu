@@ -295,27 +295,26 @@ int run_m5(dw_lattice *lat, int prec, void *out, const void *in, long long nsite
   return DW_OK;
 }
 
-// Tile of the checkerboard stencil: two slices per thread where Ls allows,
-// 32-site tiles, the register variant (capped at FP32 / FP16), and but for D^+ at
-// FP32 / FP16 the slice groups split over three (else two) CTAs, as the tuner
-// prefers on the full lattice (D^+ keeps all slices in one CTA).
+// Tile of the checkerboard stencil, by the rules of the full lattice (register_tile): two
+// slices per thread where Ls allows (FP64 one but for D^+), 32-site tiles, the register
+// variant (capped at FP32 / FP16), CTAs of two slice groups (FP64 up to four; D^+ at FP32 /
+// FP16 all of them).
 // Key of a tuned checkerboard tile in the lattice's tile map (its own op codes).
 constexpr int kCbOpKey = 16;
 
 TileConfig cb_default_tile(const dw_lattice *lat, int prec, int op) {
   TileConfig t;
-  t.spt = lat->Ls % 2 == 0 ? 2 : 1;
+  const bool f64 = prec == DW_F64;
+  t.spt = lat->Ls % 2 == 0 && !(f64 && op != OP_DDAG) ? 2 : 1;
   t.tx = 32;
-  t.variant = prec == DW_F64 ? 0 : 4;
+  t.variant = f64 ? 0 : 4;
   t.zblk = auto_zblk(lat, prec);
   const int nchunk = lat->Ls / t.spt;
-  t.sgrp = 1;
-  if (op != OP_DDAG && prec != DW_F64)
-    for (int g : {3, 2})
-      if (nchunk % g == 0) {
-        t.sgrp = g;
-        break;
-      }
+  int cpc = nchunk;
+  if (f64 || op != OP_DDAG)
+    for (cpc = f64 ? 4 : 2; nchunk % cpc;) --cpc;
+  t.sgrp = nchunk / cpc;
+  if (op == OP_DDAG && t.sgrp > 8) t.sgrp = 1;
   return t;
 }
 
