@@ -84,6 +84,8 @@ _lock = threading.Lock()
 def load_library():
     """Load the in-tree CUDA library; raises if it has not been built."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -141,6 +143,8 @@ def load_library():
 
 
 def _check(rc, allow=()):
+    if rc == 0:
+        return rc
     if rc < 0 and rc not in allow:
         msg = load_library().dw_last_error().decode(errors="replace")
         raise DWError(rc, msg)
