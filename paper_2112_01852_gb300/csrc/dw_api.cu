@@ -142,8 +142,9 @@ TileConfig register_tile(const dw_lattice *lat, int prec, int op, int nrhs) {
 
 // Untuned choice: the register tile, or where it was faster
 //  - Dhop at FP32 / FP16 (and D at FP16): the rows of a tile staged in shared memory
-//    (variant 6) where planes and Ls allow tiles of 64 sites or more, Dhop with two slices
-//    per CTA and the widest tile of 128, 96 and 64 sites, D with 64 sites and two groups;
+//    (variant 6) where planes and Ls allow tiles of 64 sites or more, Dhop at FP32 with two
+//    slices per CTA and the widest tile of 128, 96 and 64 sites, FP16 with 64 sites and two
+//    groups (24^3 x 48 x 8 Dhop 277 -> 262 us);
 //  - D at FP32, and at an odd multiple of three slices: three or four slices per thread
 //    uncapped (variant 3: its loads of the s-neighbours shared by more slices);
 //  - an odd Ls at FP16: the prefetch variant 3;
@@ -172,7 +173,8 @@ TileConfig default_tile(const dw_lattice *lat, int prec, int op, int nrhs) {
     t.variant = 3;
   } else if (op != OP_DDAG && !(op == OP_D && prec == DW_F32) && plane % 32 == 0) {
     t.variant = 6;
-    t.tx = op == OP_D ? 64 : (nblk % 4 == 0 ? 128 : (nblk % 3 == 0 ? 96 : 64));
+    t.tx = nblk % 4 == 0 ? 128 : (nblk % 3 == 0 ? 96 : 64);
+    if (op == OP_D || (prec == DW_F16 && nblk % 2 == 0)) t.tx = 64;
     t.sgrp = (Ls / 2) / largest_divisor(Ls / 2, op == OP_D || t.tx == 64 ? 2 : 1);
   }
   return tile_valid(lat, prec, op, t) ? t : base;
