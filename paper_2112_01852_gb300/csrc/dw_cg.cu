@@ -137,11 +137,17 @@ struct Solve {
   }
 
   // Reliable update of every RHS flagged need_update (first: initial residual).
-  int reliable(void *x, const void *b, int first) {
+  // x_zero: the start vector is zero, so A x needs no operator.
+  int reliable(void *x, const void *b, int first, bool x_zero = false) {
     if (!first && cg_accumulate_x(c, pr, x, w->xs, w->state, st))
       return cuda_fail(cudaGetLastError(), "accumulate launch");
     int rc;
-    if (eo) {
+    if (x_zero) {
+      const size_t bytes = eo ? cb_field_bytes(lat, DW_F64, nrhs) : field_bytes(lat, DW_F64, nrhs);
+      if (cudaMemsetAsync(w->Ax64, 0, bytes, st) != cudaSuccess)
+        return cuda_fail(cudaGetLastError(), "residual memset");
+      rc = DW_OK;
+    } else if (eo) {
       rc = apply_schur(lat, DW_F64, w->tmp64, x, mf, nrhs, false, w->e1_64, w->e2_64, st,
                        gate_update(), kCGStateInts, nullptr);
       if (rc) return rc;
@@ -212,7 +218,7 @@ int cg_run(dw_lattice *lat, void *x, const void *b, const double *mf, int nrhs, 
       (rc = ensure(&w->rs, &w->rs_cap, fpr)) || (rc = ensure(&w->xs, &w->xs_cap, fpr)) ||
       (rc = ensure((void **)&w->partials, &w->partials_cap,
                    sizeof(double) * (size_t)S.c.nblk * nrhs)) ||
-      (rc = ensure((void **)&w->sums, &w->sums_cap, sizeof(double) * nrhs)) ||
+      (rc = ensure((void **)&w->sums, &w->sums_cap, sizeof(double) * 2 * nrhs)) ||
       (rc = ensure((void **)&w->state, &w->state_cap, sizeof(CGState) * nrhs)))
     return rc;
   if (eo && ((rc = ensure(&w->e1, &w->e1_cap, fpp)) || (rc = ensure(&w->e2, &w->e2_cap, fpp)) ||
@@ -222,12 +228,14 @@ int cg_run(dw_lattice *lat, void *x, const void *b, const double *mf, int nrhs, 
   cudaStream_t st = w->stream;
 
 
-  // |b| per RHS
-  std::vector<double> b2(nrhs);
+  // |b| and |x0| per RHS
+  std::vector<double> b2(2 * nrhs);
   if (blas_redot(S.c, DW_F64, b, DW_F64, b, w->partials, nullptr, st) ||
-      blas_finalize_sum(S.c, w->partials, w->sums, st))
+      blas_finalize_sum(S.c, w->partials, w->sums, st) ||
+      blas_redot(S.c, DW_F64, x, DW_F64, x, w->partials, nullptr, st) ||
+      blas_finalize_sum(S.c, w->partials, w->sums + nrhs, st))
     return cuda_fail(cudaGetLastError(), "norm launch");
-  e = cudaMemcpyAsync(b2.data(), w->sums, sizeof(double) * nrhs, cudaMemcpyDeviceToHost, st);
+  e = cudaMemcpyAsync(b2.data(), w->sums, sizeof(double) * 2 * nrhs, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_fail(e, "norm readback");
 
@@ -277,7 +285,9 @@ int cg_run(dw_lattice *lat, void *x, const void *b, const double *mf, int nrhs, 
   }
 
   // initial residual
-  if ((rc = S.reliable(x, b, 1))) return rc;
+  bool x_zero = true;
+  for (int r = 0; r < nrhs; ++r) x_zero &= b2[nrhs + r] == 0.0;
+  if ((rc = S.reliable(x, b, 1, x_zero))) return rc;
   // even-odd: one extra pass of the inner operator (its result is recomputed by
   // the first iteration) so that every
   // kernel it launches has been set up before the stream is captured
