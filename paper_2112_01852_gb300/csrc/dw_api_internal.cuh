@@ -146,6 +146,8 @@ int run_dslash_cb(dw_lattice *lat, int prec, int op, void *out, const void *nbr,
                   double *norm_partials, const TileConfig *force = nullptr,
                   const ResidualFuse *fuse = nullptr);
 long long cb_ctas_per_rhs(const dw_lattice *lat, int prec, int op);
+// Whether apply_schur at `prec` launches checkerboard op `op`.
+bool cb_op_used(const dw_lattice *lat, int prec, int op);
 // Time the checkerboard tiles of (prec, op) once per lattice and keep the best.
 int tune_cb(dw_lattice *lat, int prec, int op, cudaStream_t st);
 // out_o = Dhat in_o or Dhat^+ in_o; t1, t2 even scratch fields

@@ -265,8 +265,8 @@ int cg_run(dw_lattice *lat, void *x, const void *b, const double *mf, int nrhs, 
   // tile choice for the inner operator of this solve (timed once per lattice
   // and RHS count, then cached; the FP64 operator of the reliable updates keeps
   // the untuned tile unless it is the inner operator)
-  for (int op : {(int)OP_D, (int)OP_DDAG, (int)OP_HOP_LOCAL}) {
-    if (eo && (S.pp != DW_F64 || op != OP_D))  // (the FP64 Dhat has no fused D hop)
+  for (int op : {(int)OP_D, (int)OP_DDAG, (int)OP_HOP_LOCAL, (int)OP_D_M5, (int)OP_HOP_DAG_M5}) {
+    if (eo && cb_op_used(lat, S.pp, op))
       rc = tune_cb(lat, S.pp, op, st);
     else if (eo || op > OP_DDAG)
       continue;

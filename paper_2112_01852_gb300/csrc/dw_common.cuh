@@ -200,13 +200,17 @@ __host__ __device__ __forceinline__ long long link_off(int x4, int mu, int nlv) 
 //                      streaming pass, phi_kernel in dw_eo.cu): local term of `own` plus
 //                      hscale * b * Dhop in
 //   OP_HOP_SCALED_DAG  hscale * b * Dhop^+ in, no local term
+//   OP_D_M5            (1 + (c/b) K) A^-1 of hscale Dhop (b + cK) in (checkerboard)
+//   OP_HOP_DAG_M5      (1 + (c/b) K^+) A^-+ of hscale b Dhop^+ in (checkerboard)
 enum OpKind {
   OP_DHOP = 0,
   OP_DHOP_DAG = 1,
   OP_D = 2,
   OP_DDAG = 3,
   OP_HOP_LOCAL = 4,
-  OP_HOP_SCALED_DAG = 5
+  OP_HOP_SCALED_DAG = 5,
+  OP_D_M5 = 6,
+  OP_HOP_DAG_M5 = 7
 };
 
 struct DslashParams {

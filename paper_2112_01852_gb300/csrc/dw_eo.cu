@@ -311,11 +311,21 @@ TileConfig cb_default_tile(const dw_lattice *lat, int prec, int op) {
   t.zblk = auto_zblk(lat, prec);
   const int nchunk = lat->Ls / t.spt;
   int cpc = nchunk;
-  if (f64 || op != OP_DDAG)
+  const bool m5 = op == OP_D_M5 || op == OP_HOP_DAG_M5;
+  if (!m5 && (f64 || op != OP_DDAG))
     for (cpc = f64 ? 4 : 2; nchunk % cpc;) --cpc;
   t.sgrp = nchunk / cpc;
   if (op == OP_DDAG && t.sgrp > 8) t.sgrp = 1;
   return t;
+}
+
+// The M5 forms take all slice groups of a tile into one CTA: at most eight (256 threads at
+// 128 registers, two CTAs on an SM, their slices in 2 x 48 KB of shared memory).  Nine
+// groups, or three CTAs of three as a cluster, lost to the pass of its own (20^4 x 9 FP32
+// 392 -> 464 us).
+bool m5_fits(const dw_lattice *lat, int prec) {
+  const TileConfig t = cb_default_tile(lat, prec, OP_D_M5);
+  return lat->Ls / t.spt <= 8;
 }
 
 TileConfig cb_tile(const dw_lattice *lat, int prec, int op) {
@@ -445,11 +455,21 @@ int apply_schur(dw_lattice *lat, int prec, void *out, const void *in, const doub
   const double alpha = lat->b * (4.0 - lat->M5) + 1.0;
   const double beta = lat->c * (4.0 - lat->M5) - 1.0;
   int rc;
+  // FP32 / FP16: the A^-1 pass rides in the hop before it (the M5 forms) where all slices
+  // of a site fit a CTA; t1 is then not used
+  const bool fused = prec != DW_F64 && m5_fits(lat, prec);
+  if (fused) {
+    const double h = -0.5;
+    if ((rc = run_dslash_cb(lat, prec, dag ? OP_HOP_DAG_M5 : OP_D_M5, t2, in, nullptr, 0, alpha,
+                            beta, h, mf, nrhs, st, gate, gate_stride, nullptr)))
+      return rc;
+  }
   if (dag) {
     // t1 = -b/2 Dhop^+ in on even sites, t2 = (1 + (c/b) K^+) A^-+ t1
-    if ((rc = run_dslash_cb(lat, prec, OP_HOP_SCALED_DAG, t1, in, nullptr, 0, 0.0, 0.0, -0.5, mf,
+    if (!fused && ((rc = run_dslash_cb(lat, prec, OP_HOP_SCALED_DAG, t1, in, nullptr, 0, 0.0, 0.0, -0.5, mf,
                             nrhs, st, gate, gate_stride, nullptr)) ||
-        (rc = apply_m5_inv_phi(lat, prec, t2, t1, mf, nrhs, true, st, gate, gate_stride)))
+                   (rc = apply_m5_inv_phi(lat, prec, t2, t1, mf, nrhs, true, st, gate,
+                                          gate_stride))))
       return rc;
     // out = A^+ in - H_eo^+ t2 on odd sites
     return run_dslash_cb(lat, prec, OP_DDAG, out, t2, in, 1, alpha, beta, 0.5, mf, nrhs, st, gate,
@@ -461,15 +481,26 @@ int apply_schur(dw_lattice *lat, int prec, void *out, const void *in, const doub
         (rc = run_dslash_cb(lat, prec, OP_HOP_LOCAL, t1, out, nullptr, 0, 0.0, 0.0, -0.5, mf, nrhs,
                             st, gate, gate_stride, nullptr)))
       return rc;
-  } else if ((rc = run_dslash_cb(lat, prec, OP_D, t1, in, nullptr, 0, 0.0, 0.0, -0.5, mf, nrhs, st,
-                                 gate, gate_stride, nullptr))) {
+  } else if (!fused && (rc = run_dslash_cb(lat, prec, OP_D, t1, in, nullptr, 0, 0.0, 0.0, -0.5, mf,
+                                           nrhs, st, gate, gate_stride, nullptr))) {
     return rc;
   }
   // t2 = (1 + (c/b) K) A^-1 t1, out = A in - H_oe A^-1 t1 on odd sites
-  if ((rc = apply_m5_inv_phi(lat, prec, t2, t1, mf, nrhs, false, st, gate, gate_stride)))
+  if (!fused &&
+      (rc = apply_m5_inv_phi(lat, prec, t2, t1, mf, nrhs, false, st, gate, gate_stride)))
     return rc;
   return run_dslash_cb(lat, prec, OP_HOP_LOCAL, out, t2, in, 1, alpha, beta, 0.5, mf, nrhs, st,
                        gate, gate_stride, norm_partials);
+}
+
+bool cb_op_used(const dw_lattice *lat, int prec, int op) {
+  const bool fused = prec != DW_F64 && m5_fits(lat, prec);
+  switch (op) {
+    case OP_D: return prec != DW_F64 && !fused;
+    case OP_D_M5:
+    case OP_HOP_DAG_M5: return fused;
+  }
+  return op == OP_DDAG || op == OP_HOP_LOCAL;
 }
 
 // Times the checkerboard tiles of (prec, op) on two scratch parity fields (the
@@ -499,9 +530,10 @@ int tune_cb(dw_lattice *lat, int prec, int op, cudaStream_t st) {
     for (int tx : {32, 64, 96, 128})
       for (int sgrp : {1, 2, 3, 4, 6}) {
         if (lat->Ls % spt || (lat->Ls / spt) % sgrp || (op == OP_DDAG && sgrp > 8)) continue;
+        if ((op == OP_D_M5 || op == OP_HOP_DAG_M5) && (tx > 64 || sgrp > 1)) continue;
         const TileConfig t{spt, tx, prec == DW_F64 ? 0 : 4, za, sgrp};
         if (tx * (lat->Ls / spt / sgrp) > 1024) continue;
-        if (run_dslash_cb(lat, prec, op, lat->stage_out, lat->stage_in, nullptr, 0, 0.0, 0.0,
+        if (run_dslash_cb(lat, prec, op, lat->stage_out, lat->stage_in, nullptr, 0, 4.0, 0.5,
                           -0.5, &mf, 1, st, nullptr, 0, nullptr, &t)) {
           cudaGetLastError();
           continue;  // not launchable (CTA limits)
@@ -509,7 +541,7 @@ int tune_cb(dw_lattice *lat, int prec, int op, cudaStream_t st) {
         float ms[2];
         for (float &m : ms) {
           cudaEventRecord(e0, st);
-          run_dslash_cb(lat, prec, op, lat->stage_out, lat->stage_in, nullptr, 0, 0.0, 0.0, -0.5,
+          run_dslash_cb(lat, prec, op, lat->stage_out, lat->stage_in, nullptr, 0, 4.0, 0.5, -0.5,
                         &mf, 1, st, nullptr, 0, nullptr, &t);
           cudaEventRecord(e1, st);
           cudaEventSynchronize(e1);
