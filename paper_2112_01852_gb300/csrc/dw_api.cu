@@ -127,7 +127,9 @@ static int largest_divisor(int n, int cap) {
 // times the best.
 TileConfig register_tile(const dw_lattice *lat, int prec, int op, int nrhs) {
   const int Ls = lat->Ls;
-  if (lat->cplx && prec == DW_F32) return generic_tile(lat, prec, op);
+  // (an Ls that fits no CTA there is refused here too; dw_set_tile and dw_tune split it)
+  const TileConfig gen = generic_tile(lat, prec, op);
+  if ((lat->cplx && prec == DW_F32) || !tile_valid(lat, prec, op, gen)) return gen;
   const bool f64 = prec == DW_F64, even = Ls % 2 == 0;
   int spt = even ? 2 : (op == OP_DDAG && Ls % 3 == 0 ? 3 : 1);
   if (f64 ? op != OP_DDAG : even && lat->V5 * nrhs <= 64LL * 8 * lat->num_sms) spt = 1;
@@ -137,7 +139,7 @@ TileConfig register_tile(const dw_lattice *lat, int prec, int op, int nrhs) {
   // several RHS: one sweep after another (see dw_tune), each with its own reuse window
   const TileConfig t{spt,  32, f64 ? 0 : 4, auto_zblk(lat, prec), nchunk / cpc,
                      nrhs > 1 && !f64 ? 1 : 0};
-  return tile_valid(lat, prec, op, t) ? t : generic_tile(lat, prec, op);
+  return tile_valid(lat, prec, op, t) ? t : gen;
 }
 
 // Untuned choice: the register tile, or where it was faster
@@ -146,9 +148,10 @@ TileConfig register_tile(const dw_lattice *lat, int prec, int op, int nrhs) {
 //    slices per CTA and the widest tile of 128, 96 and 64 sites, FP16 with 64 sites and two
 //    groups (24^3 x 48 x 8 Dhop 277 -> 262 us);
 //  - D at FP32, and at an odd multiple of three slices: three or four slices per thread
-//    uncapped (variant 3: its loads of the s-neighbours shared by more slices);
-//  - an odd Ls at FP16: the prefetch variant 3;
-//  - Dhop at FP64: the prefetch variant 2 (16^4 x 16 1.65 -> 1.53 ms).
+//    uncapped (variant 2, whose D is the register path: its loads of the s-neighbours
+//    shared by more slices);
+//  - an odd Ls at FP16, and Dhop at FP64: the prefetch variant 2 (FP64 16^4 x 16 1.65 -> 1.53
+//    ms).
 // All of them sum the hops in the same order: the choice does not change a result.
 TileConfig default_tile(const dw_lattice *lat, int prec, int op, int nrhs) {
   const TileConfig base = register_tile(lat, prec, op, nrhs);
@@ -164,13 +167,13 @@ TileConfig default_tile(const dw_lattice *lat, int prec, int op, int nrhs) {
   const int plane = lat->dims[0] * lat->dims[1], nblk = plane / 32;
   const int blocks = (plane + 31) / 32;  // 32-site tiles of a plane
   if (op == OP_D && (prec == DW_F32 || Ls % 2) && (Ls % 3 == 0 || Ls % 4 == 0)) {
-    t.variant = 3;
+    t.variant = 2;
     t.spt = Ls % 3 == 0 ? 3 : 4;
     t.tx = Ls % 2 == 0 && (blocks % 2 == 0 || blocks >= 20) ? 64 : 32;
     t.sgrp = (Ls / t.spt) / largest_divisor(Ls / t.spt, Ls % 2 == 0 ? 2 : 1);
   } else if (Ls % 2) {
     if (prec == DW_F32 || (op == OP_DDAG && Ls % 3 == 0)) return base;
-    t.variant = 3;
+    t.variant = 2;
   } else if (op != OP_DDAG && !(op == OP_D && prec == DW_F32) && plane % 32 == 0) {
     t.variant = 6;
     t.tx = nblk % 4 == 0 ? 128 : (nblk % 3 == 0 ? 96 : 64);
