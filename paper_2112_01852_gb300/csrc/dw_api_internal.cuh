@@ -75,7 +75,7 @@ int tune_tile(dw_lattice *lat, int prec, int op, int nrhs, cudaStream_t st, bool
 // Stencil launch (op = OpKind) at precision `prec` over nrhs RHS; mf_host may be
 // NULL for the hopping-only kinds; `force` overrides the tile choice.
 // `gate` (optional) skips the CTAs of RHS r unless gate[r * gate_stride] != 0;
-// halo_up / halo_dn (optional, variant 0 tiles only) replace the t-neighbours
+// halo_up / halo_dn (optional, tiles of variants 0 and 4 only) replace the t-neighbours
 // at the t faces of a decomposed sub-lattice; norm_partials (optional, OP_D
 // only) receives |out|^2 per CTA, [rhs][dslash_ctas_per_rhs]; t_begin / t_count
 // restrict the output to the time slices t_begin .. t_begin + t_count - 1

@@ -227,8 +227,8 @@ struct DslashParams {
   const int *gate;      // optional: CTAs of RHS r run only if gate[r * gate_stride] != 0
   int gate_stride;
   double *norm_partials;  // optional (OP_D): |out|^2 per CTA at [rhs][CTA index in the RHS]
-  const void *halo_up;  // optional t-face halves from the rank above (variant 0 only)
-  const void *halo_dn;  // optional t-face halves from the rank below (variant 0 only)
+  const void *halo_up;  // optional t-face halves from the rank above (variants 0 and 4 only)
+  const void *halo_dn;  // optional t-face halves from the rank below (variants 0 and 4 only)
   int tiles_per_plane;  // set by the launcher: CTAs per (x, y) plane
   int zblk;             // set by the launcher: z-blocks of the traversal order
   int sgrp;             // set by the launcher: CTAs per site tile (slice groups)
