@@ -151,13 +151,15 @@ int dw_apply_DdagD_noalloc(dw_lattice *lat, void *out, const void *in, const dou
  * the lattice precision: copies in to the device, applies, copies out back and
  * returns when the output is in out_host.  Device staging buffers are
  * lattice-owned.  mf may be NULL for DW_OP_DHOP / DW_OP_DHOP_DAG.
- * When Lx*Ly*Lz is a multiple of 32 the field moves in t slabs (up to 16, each
+ * When Lx*Ly*Lz is a multiple of 32 the field moves in t slabs (up to 64, each
  * of at least 8192 4D sites): the copy in of one slab, the operator on the
  * previous one (once its t neighbours are resident) and the copy out of the
  * one before run at the same time, on `stream` and two lattice-owned streams.
  * Pinned host buffers (cudaHostAlloc / cudaHostRegister) are needed for the
  * copies to overlap; pageable ones work but serialise.  out_host must not
- * overlap in_host.
+ * overlap in_host.  Returns DW_ERR_TIMEOUT (out_host may then be wrong) when a
+ * stencil launch on this lattice gave up a bounded wait since the last
+ * dw_device_status; the word is then cleared.
  */
 int dw_apply_host(dw_lattice *lat, int op, void *out_host, const void *in_host,
                   const double *mf, int nrhs, void *stream);
@@ -296,10 +298,13 @@ int dw_get_tile(dw_lattice *lat, int op, int prec, int nrhs, int *spt, int *tx, 
 
 /*
  * Device-side status of the lattice's kernels.  Kernels that wait for their own
- * asynchronous copies (stencil variant 6) bound every wait; one that gives up
- * sets a lattice-owned device word and returns without finishing (its output is
- * then wrong).  This call synchronises the device, reads and clears the word and
- * returns DW_OK or DW_ERR_TIMEOUT.
+ * asynchronous copies (stencil variants 6 and 7; untuned launches of Dhop and
+ * Dhop^+ at DW_F32 / DW_F16 and of D at DW_F16 take variant 6 where the lattice
+ * allows) bound every wait; one that gives up sets a lattice-owned device word
+ * and goes on, and its output may then be wrong.  dw_apply_Dhop and its like
+ * return before the kernels have run and cannot report that: this call
+ * synchronises the device, reads and clears the word and returns DW_OK or
+ * DW_ERR_TIMEOUT.
  */
 int dw_device_status(dw_lattice *lat);
 
@@ -328,7 +333,7 @@ int dw_set_complex_layout(dw_lattice *lat, int interleaved);
  * (6, 7) on this lattice: polls >= 0 lets that wait give up after `polls`
  * polls of the barrier, -1 (the default) restores the built-in bound of about a
  * second.  A wait that gives up sets the lattice's status word (reported by
- * dw_device_status, and by dw_cg_solve / dw_solve_eo as DW_ERR_TIMEOUT); the
+ * dw_device_status, and by dw_apply_host / dw_cg_solve / dw_solve_eo as DW_ERR_TIMEOUT); the
  * kernel then waits once more, with the built-in bound, for the copies it
  * issued, so that it never reads or refills a slot with a copy in flight.
  * polls = 0 therefore exercises the timeout report without losing the result:

@@ -29,6 +29,7 @@ struct dw_lattice {
   int num_sms;
   bool gauge_loaded;
   int *dev_status;  // device word the kernels set when a bounded wait gives up
+  int *host_status;  // pinned copy of it that dw_apply_host reads (created on first use)
   int wait_polls;   // dw_set_wait_polls (-1: the kernels' built-in bound)
   bool cplx;        // dw_set_complex_layout: FP32 fields hold interleaved-complex quads
   double reliable_delta;  // dw_set_reliable_delta (0: the solvers' defaults)

@@ -113,6 +113,31 @@ std::vector<Task> schedule(int n, int passes) {
   return all;
 }
 
+// The lattice's status word, copied on `st` behind its launches into a pinned word (the
+// caller synchronises `st` before it looks).
+cudaError_t status_copy(dw_lattice *lat, cudaStream_t st) {
+  if (!lat->host_status) {
+    const cudaError_t e = cudaHostAlloc((void **)&lat->host_status, sizeof(int), 0);
+    if (e != cudaSuccess) {
+      lat->host_status = nullptr;
+      return e;
+    }
+  }
+  return cudaMemcpyAsync(lat->host_status, lat->dev_status, sizeof(int), cudaMemcpyDeviceToHost,
+                         st);
+}
+
+// The call's last step, everything on `st` being done: a stencil launch that gave up a
+// bounded wait has set the word, and the output may be wrong; report it once.
+int status_result(dw_lattice *lat, cudaStream_t st) {
+  if (!*lat->host_status) return DW_OK;
+  cudaError_t e = cudaMemsetAsync(lat->dev_status, 0, sizeof(int), st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) return cuda_fail(e, "status clear");
+  return fail(DW_ERR_TIMEOUT,
+              "a stencil kernel gave up waiting for its shared-memory copies");
+}
+
 }  // namespace
 
 int apply_host_pipelined(dw_lattice *lat, int op, void *out_host, const void *in_host,
@@ -139,8 +164,10 @@ int apply_host_pipelined(dw_lattice *lat, int op, void *out_host, const void *in
     if (rc) return rc;
     e = cudaMemcpyAsync(out_host, lat->stage_out, bytes, cudaMemcpyDeviceToHost, st);
     if (e != cudaSuccess) return cuda_fail(e, "device-to-host copy");
+    const cudaError_t es = status_copy(lat, st);
     e = cudaStreamSynchronize(st);
-    return e == cudaSuccess ? DW_OK : cuda_fail(e, "stream synchronize");
+    if (e == cudaSuccess) e = es;
+    return e == cudaSuccess ? status_result(lat, st) : cuda_fail(e, "stream synchronize");
   }
   rc = pipe_streams(lat);
   if (rc) return rc;
@@ -201,9 +228,11 @@ int apply_host_pipelined(dw_lattice *lat, int op, void *out_host, const void *in
       if (e != cudaSuccess) return bail(cuda_fail(e, "device-to-host copy"));
     }
   }
+  e = status_copy(lat, st);
+  if (e != cudaSuccess) return bail(cuda_fail(e, "status copy"));
   e = cudaStreamSynchronize(lat->pipe_out);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  return e == cudaSuccess ? DW_OK : cuda_fail(e, "stream synchronize");
+  return e == cudaSuccess ? status_result(lat, st) : cuda_fail(e, "stream synchronize");
 }
 
 void pipe_release(dw_lattice *lat) {
@@ -211,6 +240,8 @@ void pipe_release(dw_lattice *lat) {
   lat->pipe_events.clear();
   if (lat->pipe_in) cudaStreamDestroy(lat->pipe_in);
   if (lat->pipe_out) cudaStreamDestroy(lat->pipe_out);
+  if (lat->host_status) cudaFreeHost(lat->host_status);
+  lat->host_status = nullptr;
   lat->pipe_in = lat->pipe_out = nullptr;
 }
 
