@@ -503,8 +503,8 @@ bool cb_op_used(const dw_lattice *lat, int prec, int op) {
   return op == OP_DDAG || op == OP_HOP_LOCAL;
 }
 
-// Times the checkerboard tiles of (prec, op) on two scratch parity fields (the
-// hopping-only form, one RHS) and keeps the fastest for later launches.
+// Times the untuned checkerboard tile of (prec, op) and a list of others on two scratch
+// parity fields (the hopping-only form, one RHS) and keeps the fastest for later launches.
 int tune_cb(dw_lattice *lat, int prec, int op, cudaStream_t st) {
   if (lat->tuned.count(std::make_tuple(prec, kCbOpKey + op, 0))) return DW_OK;
   const size_t bytes = cb_field_bytes(lat, prec, 1);
@@ -523,8 +523,31 @@ int tune_cb(dw_lattice *lat, int prec, int op, cudaStream_t st) {
     cudaEventDestroy(e0);
     return cuda_fail(cudaGetLastError(), "event");
   }
-  TileConfig best_t = cb_default_tile(lat, prec, op);
-  float best = 1e30f;
+  auto launch = [&](int o, const TileConfig &t) {
+    return run_dslash_cb(lat, prec, o, lat->stage_out, lat->stage_in, nullptr, 0, 4.0, 0.5, -0.5,
+                         &mf, 1, st, nullptr, 0, nullptr, &t);
+  };
+  // the faster of two launches (1e30: the tile does not launch)
+  auto time_tile = [&](const TileConfig &t) {
+    float best_ms = 1e30f;
+    if (launch(op, t)) {
+      cudaGetLastError();
+      return best_ms;  // CTA limits
+    }
+    for (int r = 0; r < 2; ++r) {
+      cudaEventRecord(e0, st);
+      launch(op, t);
+      cudaEventRecord(e1, st);
+      cudaEventSynchronize(e1);
+      float m = 1e30f;
+      if (cudaEventElapsedTime(&m, e0, e1) == cudaSuccess) best_ms = std::min(best_ms, m);
+    }
+    return best_ms;
+  };
+  // the untuned tile is the one to beat: its slice groups need not be in the list below
+  const TileConfig untuned = cb_default_tile(lat, prec, op);
+  TileConfig best_t = untuned;
+  float best = time_tile(best_t);
   const int za = auto_zblk(lat, prec);
   for (int spt : {1, 2, 3, 4})
     for (int tx : {32, 64, 96, 128})
@@ -533,26 +556,14 @@ int tune_cb(dw_lattice *lat, int prec, int op, cudaStream_t st) {
         if ((op == OP_D_M5 || op == OP_HOP_DAG_M5) && (tx > 64 || sgrp > 1)) continue;
         const TileConfig t{spt, tx, prec == DW_F64 ? 0 : 4, za, sgrp};
         if (tx * (lat->Ls / spt / sgrp) > 1024) continue;
-        if (run_dslash_cb(lat, prec, op, lat->stage_out, lat->stage_in, nullptr, 0, 4.0, 0.5,
-                          -0.5, &mf, 1, st, nullptr, 0, nullptr, &t)) {
-          cudaGetLastError();
-          continue;  // not launchable (CTA limits)
-        }
-        float ms[2];
-        for (float &m : ms) {
-          cudaEventRecord(e0, st);
-          run_dslash_cb(lat, prec, op, lat->stage_out, lat->stage_in, nullptr, 0, 4.0, 0.5, -0.5,
-                        &mf, 1, st, nullptr, 0, nullptr, &t);
-          cudaEventRecord(e1, st);
-          cudaEventSynchronize(e1);
-          m = 1e30f;
-          if (cudaEventElapsedTime(&m, e0, e1) != cudaSuccess) m = 1e30f;
-        }
-        if (std::min(ms[0], ms[1]) < best) {
-          best = std::min(ms[0], ms[1]);
+        const float ms = time_tile(t);
+        if (ms < best) {
+          best = ms;
           best_t = t;
         }
       }
+  // again beside the winner: the first timing may have met rising clocks
+  if (time_tile(untuned) <= time_tile(best_t)) best_t = untuned;
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   clear_error();
