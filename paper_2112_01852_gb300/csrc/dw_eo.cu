@@ -530,9 +530,9 @@ int tune_cb(dw_lattice *lat, int prec, int op, cudaStream_t st) {
   // the faster of two launches (1e30: the tile does not launch)
   auto time_tile = [&](const TileConfig &t) {
     float best_ms = 1e30f;
-    if (launch(op, t)) {
+    if (launch(op, t) || (op == OP_HOP_LOCAL && launch(OP_HOP_SCALED_DAG, t))) {
       cudaGetLastError();
-      return best_ms;  // CTA limits
+      return best_ms;  // CTA limits (of either hop that runs on this tile, see cb_tile)
     }
     for (int r = 0; r < 2; ++r) {
       cudaEventRecord(e0, st);
