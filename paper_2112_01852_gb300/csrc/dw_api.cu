@@ -60,6 +60,15 @@ int ensure_buffer(void **buf, size_t *cap, size_t need) {
   return DW_OK;
 }
 
+// Scope in which the calling thread may allocate although another thread, or this one on
+// another stream, is capturing a graph: creating a pool and allocating from it have nothing
+// to do with that capture, but in its (default) global mode they would invalidate it.
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 PhiScratch::PhiScratch(dw_lattice *lat, int op, int prec, int nrhs, cudaStream_t st_) : st(st_) {
   if (op != OP_D || prec != DW_F64 || lat->V5 * nrhs < kPhiPassMinSites) return;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -68,6 +77,7 @@ PhiScratch::PhiScratch(dw_lattice *lat, int op, int prec, int nrhs, cudaStream_t
     return;
   }
   const size_t need = field_bytes(lat, prec, nrhs);
+  const RelaxedCapture relaxed;
   cudaMemPool_t pool;
   {
     std::lock_guard<std::mutex> g(lat->pool_lock);
@@ -94,6 +104,12 @@ PhiScratch::PhiScratch(dw_lattice *lat, int op, int prec, int nrhs, cudaStream_t
     cudaGetLastError();
     p = nullptr;
   }
+}
+
+PhiScratch::~PhiScratch() {
+  if (!p) return;
+  const RelaxedCapture relaxed;
+  cudaFreeAsync(p, st);
 }
 
 // z-blocks of the traversal order: the fewest that keep the t-reuse window of

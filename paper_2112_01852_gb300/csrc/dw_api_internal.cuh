@@ -97,9 +97,7 @@ struct PhiScratch {
   void *p = nullptr;
   cudaStream_t st;
   PhiScratch(dw_lattice *lat, int op, int prec, int nrhs, cudaStream_t st_);
-  ~PhiScratch() {
-    if (p) cudaFreeAsync(p, st);
-  }
+  ~PhiScratch();
   PhiScratch(const PhiScratch &) = delete;
   PhiScratch &operator=(const PhiScratch &) = delete;
 };

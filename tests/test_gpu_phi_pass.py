@@ -1,6 +1,8 @@
 """The FP64 D with its (b + cK) pass: bit for bit the fused kernel, which a capturing
 stream takes (no allocation there), and within the oracle's tolerance."""
 
+import threading
+
 import numpy as np
 import pytest
 
@@ -43,3 +45,43 @@ def test_phi_pass_equals_fused(dims, Ls, nrhs, kind):
                            for r in range(nrhs)])
     assert oracle.rel_l2(got, want) <= TOL[dw.DW_F64]
     lat.close()
+
+
+@pytest.mark.parametrize("calls", [1, 2])
+def test_phi_pass_leaves_another_streams_capture_alone(calls):
+    # The first D of a lattice creates its pool and allocates; a capture in progress on
+    # another thread (in the global mode, torch's default) must survive that.
+    dims, Ls = (8, 8, 8, 16), 8
+    U, psi = make_case(dims, Ls, 1, 13)
+    lats = [Lattice(dims, Ls, prec=dw.DW_F64) for _ in range(3)]
+    for lt in lats:
+        lt.load_gauge(U)
+    cap, lat, warm = lats
+    x = cap.pack(psi)
+    y, ref, z = (lat.empty().zero_() for _ in range(3))
+    warm.D(ref, x, 0.05)  # loads the kernels, on a lattice of its own
+    warm.dhop(z, x)
+    torch.cuda.synchronize()
+    side, errors = torch.cuda.Stream(), []
+
+    def other():
+        try:
+            with torch.cuda.stream(side):
+                for _ in range(calls):
+                    lat.D(y, x, 0.05)
+        except Exception as e:  # noqa: BLE001
+            errors.append(e)
+
+    out = cap.empty().zero_()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        cap.dhop(out, x)
+        th = threading.Thread(target=other)
+        th.start()
+        th.join()
+    assert not errors
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(y, ref) and torch.equal(out, z)
+    for lt in lats:
+        lt.close()
