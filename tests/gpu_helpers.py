@@ -85,3 +85,20 @@ def valid_tiles(Ls, txs=(32, 64, 128)):
 
 def np_rng(seed):
     return np.random.default_rng(seed)
+
+
+def launches(f, name):
+    """How many kernels whose name contains `name` f() runs (torch's profiler)."""
+    import torch
+
+    def profile(g):
+        torch.cuda.synchronize()
+        with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as p:
+            g()
+            torch.cuda.synchronize()
+        return [e.name for e in p.events()]
+
+    for _ in range(3):  # a process's first profile can come back empty
+        if profile(lambda: torch.zeros(8, device="cuda").add_(1)):
+            break
+    return sum(name in n for n in profile(f))

@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 import oracle  # noqa: E402
-from gpu_helpers import TOL, make_case  # noqa: E402
+from gpu_helpers import TOL, launches, make_case  # noqa: E402
 from paper_2112_01852_gb300 import dw  # noqa: E402
 from paper_2112_01852_gb300.lattice import Lattice  # noqa: E402
 
@@ -85,3 +85,17 @@ def test_phi_pass_leaves_another_streams_capture_alone(calls):
     assert torch.equal(y, ref) and torch.equal(out, z)
     for lt in lats:
         lt.close()
+
+
+def test_tuner_times_the_phi_pass():
+    # the tiles of an FP64 D above the threshold are compared as they run: phi, then the hop
+    dims, Ls = (8, 8, 8, 16), 8
+    U, _ = make_case(dims, Ls, 1, 14)
+    lat = Lattice(dims, Ls, prec=dw.DW_F64)
+    lat.load_gauge(U)
+    n = launches(lambda: lat.tune(dw.DW_OP_D), "phi_kernel")
+    small = Lattice((8, 8, 8, 8), 7, prec=dw.DW_F64)  # below it: the fused kernel
+    small.load_gauge(U[: small.V4])
+    assert n > 0 and launches(lambda: small.tune(dw.DW_OP_D), "phi_kernel") == 0
+    lat.close()
+    small.close()
