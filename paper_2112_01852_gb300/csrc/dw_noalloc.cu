@@ -63,7 +63,10 @@ extern "C" int dw_apply_DdagD_noalloc(dw_lattice *lat, void *out, const void *in
   // The D pass overwrites every element of the intermediate, so nothing in the
   // array needs clearing first.
   cudaStream_t st = (cudaStream_t)stream;
-  rc = run_dslash(lat, lat->prec, OP_D, scratch, in, mf, nrhs, st, nullptr);
+  // (the phi scratch of an FP64 D pass is `out`, which D^+ writes last: see dw_apply_DdagD)
+  void *phi = lat->V5 * nrhs >= kPhiPassMinSites ? out : nullptr;
+  rc = run_dslash(lat, lat->prec, OP_D, scratch, in, mf, nrhs, st, nullptr, nullptr, 0, nullptr,
+                  nullptr, nullptr, 0, 0, nullptr, phi);
   if (rc) return rc;
   return run_dslash(lat, lat->prec, OP_DDAG, out, scratch, mf, nrhs, st, nullptr);
 }

@@ -1,6 +1,7 @@
 """The FP64 D with its (b + cK) pass: bit for bit the fused kernel, which a capturing
 stream takes (no allocation there), and within the oracle's tolerance."""
 
+import ctypes
 import threading
 
 import numpy as np
@@ -99,3 +100,25 @@ def test_tuner_times_the_phi_pass():
     assert n > 0 and launches(lambda: small.tune(dw.DW_OP_D), "phi_kernel") == 0
     lat.close()
     small.close()
+
+
+def test_noalloc_ddagd_takes_the_phi_pass():
+    # `out` is free until the D^+ pass: the pass needs no allocation there
+    dims, Ls = (8, 8, 8, 16), 8
+    U, psi = make_case(dims, Ls, 1, 15)
+    lat = Lattice(dims, Ls, prec=dw.DW_F64)
+    lat.load_gauge(U)
+    x = lat.pack(psi)
+    y, ref = lat.empty().zero_(), lat.empty().zero_()
+
+    def noalloc():
+        mf = (ctypes.c_double * 1)(0.05)
+        rc = dw.load_library().dw_apply_DdagD_noalloc(
+            lat.handle, y.data_ptr(), x.data_ptr(), mf, 1,
+            torch.cuda.current_stream().cuda_stream)
+        assert rc == dw.DW_OK, dw.dw_last_error()
+
+    assert launches(noalloc, "phi_kernel") == 1
+    lat.DdagD(ref, x, 0.05)
+    assert torch.equal(y, ref)
+    lat.close()
