@@ -211,7 +211,11 @@ int dw_cg_solve(dw_lattice *lat, void *x, const void *b, const double *mf, int n
  * the lattice precision, per-RHS masses mf[nrhs] (HOST).
  * dw_apply_schur: out = Dhat in (dag: Dhat^+ in) on odd eo fields at the lattice
  * precision; the even intermediates live in lattice scratch.  out must not
- * alias in.  Stream-ordered, asynchronous.
+ * alias in.  Stream-ordered, asynchronous.  With n = Ls / 2 (Ls even) or Ls:
+ * DW_F64 takes n / k <= 8, k the largest divisor of n up to 4 (so every Ls up to
+ * 10 and every even one up to 20); DW_F32 and DW_F16 take n <= 16, where Dhat
+ * counts n / 3, else n / 2, if that divides.  DW_ERR_ARG otherwise, before anything
+ * is launched.  dw_solve_eo needs an Ls that DW_F64 takes here and in dw_apply_D.
  */
 size_t dw_fermion_bytes_eo(const dw_lattice *lat, int prec, int nrhs);
 int dw_eo_split(dw_lattice *lat, void *even, void *odd, const void *full, int prec, int nrhs,

@@ -145,6 +145,8 @@ int run_dslash_cb(dw_lattice *lat, int prec, int op, void *out, const void *nbr,
                   double *norm_partials, const TileConfig *force = nullptr,
                   const ResidualFuse *fuse = nullptr);
 long long cb_ctas_per_rhs(const dw_lattice *lat, int prec, int op);
+// DW_OK, or DW_ERR_ARG for an Ls that Dhat (dag: Dhat^+) does not take at `prec`.
+int check_cb(const dw_lattice *lat, int prec, bool dag);
 // Whether apply_schur at `prec` launches checkerboard op `op`.
 bool cb_op_used(const dw_lattice *lat, int prec, int op);
 // Time the checkerboard tiles of (prec, op) once per lattice and keep the best.

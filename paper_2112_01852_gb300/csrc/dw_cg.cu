@@ -430,6 +430,10 @@ extern "C" int dw_solve_eo(dw_lattice *lat, void *x, const void *eta, const doub
   int rc = cg_prepare(lat, x, eta, mf, nrhs, tol, maxit, mode, stats, stream);
   if (rc) return rc;
   if (!eo_ok(lat)) return fail(DW_ERR_ARG, "even-odd solves need even Lx, Ly, Lz, Lt");
+  // the FP64 operators of the residuals: Dhat and its adjoint, and D on the whole lattice
+  if ((rc = check_cb(lat, DW_F64, true))) return rc;
+  if (!tile_valid(lat, DW_F64, OP_D, pick_tile(lat, DW_F64, OP_D, nrhs)))
+    return fail(DW_ERR_ARG, "the FP64 D of the residual does not take Ls = %d", lat->Ls);
   CGWork *w = lat->cg;
   cudaStream_t st = w->stream;
   const size_t h64 = cb_field_bytes(lat, DW_F64, nrhs);

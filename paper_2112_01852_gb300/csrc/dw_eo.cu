@@ -315,7 +315,6 @@ TileConfig cb_default_tile(const dw_lattice *lat, int prec, int op) {
   if (!m5 && (f64 || op != OP_DDAG))
     for (cpc = f64 ? 4 : 2; nchunk % cpc;) --cpc;
   t.sgrp = nchunk / cpc;
-  if (op == OP_DDAG && t.sgrp > 8) t.sgrp = 1;
   return t;
 }
 
@@ -335,6 +334,27 @@ TileConfig cb_tile(const dw_lattice *lat, int prec, int op) {
 }
 
 }  // namespace
+
+// The Ls that the even-odd operators take, by their slice groups n (two slices each where Ls
+// is even).  FP64: n over CTAs of up to four groups, at most the eight CTAs of a cluster of
+// D^+.  FP32 / FP16: the 16 groups of D^+ that fit one CTA; Dhat counts them after a split
+// over three, else two CTAs.  Others are refused before anything is launched, Dhat too where
+// its own hops would fit: no operator without its adjoint at FP64, and at FP32 / FP16 the Ls
+// of the operators before their tiles were split further.
+int check_cb(const dw_lattice *lat, int prec, bool dag) {
+  const int n = lat->Ls / (lat->Ls % 2 == 0 ? 2 : 1);
+  int split = 1, limit = 16;
+  if (prec == DW_F64) {
+    int cpc = 4;
+    while (n % cpc) --cpc;
+    split = cpc;
+    limit = 8;
+  } else if (!dag) {
+    split = n % 3 == 0 ? 3 : (n % 2 == 0 ? 2 : 1);
+  }
+  if (n / split <= limit) return DW_OK;
+  return fail(DW_ERR_ARG, "checkerboard stencil unavailable for this lattice (Ls = %d)", lat->Ls);
+}
 
 // A periodic hop keeps the parity of x + y + z + t only if every extent is
 // even; the even-odd split needs that.
@@ -640,6 +660,7 @@ extern "C" int dw_apply_schur(dw_lattice *lat, void *out, const void *in, const 
   if (!lat->gauge_loaded) return fail(DW_ERR_STATE, "dw_load_gauge has not been called");
   if (lat->cplx && lat->prec == DW_F32)
     return fail(DW_ERR_STATE, "interleaved-complex FP32 fields support Dhop and Dhop^+ only");
+  if ((rc = check_cb(lat, lat->prec, dag != 0))) return rc;
   const size_t need = 2 * cb_field_bytes(lat, lat->prec, nrhs);
   if ((rc = ensure_buffer(&lat->scratch, &lat->scratch_bytes, need))) return rc;
   void *t1 = lat->scratch;
