@@ -31,7 +31,6 @@ def test_phi_pass_equals_fused(dims, Ls, nrhs, kind):
     y, ref = lat.empty(nrhs), lat.empty(nrhs)
     y.zero_()
     ref.zero_()
-    lat.D(ref, x, mfs, nrhs)  # loads the kernels before the capture
     lat.D(y, x, mfs, nrhs)
     graph = torch.cuda.CUDAGraph()
     with torch.cuda.graph(graph):
@@ -40,6 +39,9 @@ def test_phi_pass_equals_fused(dims, Ls, nrhs, kind):
     graph.replay()
     torch.cuda.synchronize()
     assert torch.equal(y, ref)
+    # the pass runs from the threshold on, and not in the captured call
+    runs = [launches(f, "phi_kernel") for f in (lambda: lat.D(y, x, mfs, nrhs), graph.replay)]
+    assert runs == [1 if lat.V5 * nrhs >= 1 << 15 else 0, 0]
     got = lat.unpack(y, nrhs)
     b, c = (1.5, 0.5) if kind == dw.DW_MOBIUS else (1.0, 0.0)
     want = np.concatenate([oracle.dw(psi[r:r + 1], U, dims, Ls, 1.8, b, c, mfs[r])
