@@ -133,7 +133,7 @@ int apply_m5(dw_lattice *lat, int prec, void *out, const void *in, const double 
 // out = (1 + (c / b) K) A^-1 in (dag: the adjoint), on parity fields
 int apply_m5_inv_phi(dw_lattice *lat, int prec, void *out, const void *in, const double *mf,
                      int nrhs, bool dag, cudaStream_t st, const int *gate, int gate_stride);
-// out = in + (c / b) K in = phi / b, on parity or whole-lattice fields
+// out = in + (c / b) K in = phi / b, on parity or whole-lattice FP64 fields
 int apply_phi(dw_lattice *lat, int prec, void *out, const void *in, bool parity_field,
               const double *mf, int nrhs, cudaStream_t st, const int *gate, int gate_stride);
 // out (parity) = alpha own + beta K own + hscale Dhop (b + cK) nbr (OP_D; OP_HOP_LOCAL
@@ -147,6 +147,9 @@ int run_dslash_cb(dw_lattice *lat, int prec, int op, void *out, const void *nbr,
 long long cb_ctas_per_rhs(const dw_lattice *lat, int prec, int op);
 // DW_OK, or DW_ERR_ARG for an Ls that Dhat (dag: Dhat^+) does not take at `prec`.
 int check_cb(const dw_lattice *lat, int prec, bool dag);
+// Whether apply_schur at `prec` takes the A^-1 step into the hop before it (and leaves its
+// scratch field t1 alone).
+bool schur_fused(const dw_lattice *lat, int prec);
 // Whether apply_schur at `prec` launches checkerboard op `op`.
 bool cb_op_used(const dw_lattice *lat, int prec, int op);
 // Time the checkerboard tiles of (prec, op) once per lattice and keep the best.

@@ -221,7 +221,8 @@ int cg_run(dw_lattice *lat, void *x, const void *b, const double *mf, int nrhs, 
       (rc = ensure((void **)&w->sums, &w->sums_cap, sizeof(double) * 2 * nrhs)) ||
       (rc = ensure((void **)&w->state, &w->state_cap, sizeof(CGState) * nrhs)))
     return rc;
-  if (eo && ((rc = ensure(&w->e1, &w->e1_cap, fpp)) || (rc = ensure(&w->e2, &w->e2_cap, fpp)) ||
+  if (eo && ((!schur_fused(lat, S.pp) && (rc = ensure(&w->e1, &w->e1_cap, fpp))) ||
+             (rc = ensure(&w->e2, &w->e2_cap, fpp)) ||
              (rc = ensure(&w->e1_64, &w->e1_64_cap, f64)) ||
              (rc = ensure(&w->e2_64, &w->e2_64_cap, f64))))
     return rc;

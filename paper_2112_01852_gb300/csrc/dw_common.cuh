@@ -319,7 +319,8 @@ int launch_dslash_cplx(const DslashParams &p, int op, TileConfig cfg, cudaStream
 inline bool cplx_variant_ok(int op, int variant) {
   return (op == OP_DHOP || op == OP_DHOP_DAG) && variant >= 4 && variant <= 7;
 }
-// Checkerboard (single-parity) stencil, OP_D / OP_DDAG forms only.
+// Checkerboard (single-parity) stencil: OP_DDAG, the hops OP_HOP_LOCAL and OP_HOP_SCALED_DAG,
+// and at FP32 / FP16 OP_D, OP_D_M5 and OP_HOP_DAG_M5.
 int launch_dslash_cb(const DslashParams &p, int prec, int op, TileConfig cfg, cudaStream_t st);
 // Largest CTA the stencil kernel (op, spt, variant) can launch (0: none).
 int dslash_max_threads(int prec, int op, int spt, int variant);

@@ -2072,7 +2072,10 @@ template <class P, int VAR>
 int launch_variant_cb(const DslashParams &p, int op, TileConfig cfg, cudaStream_t st) {
   if (cfg.spt < 1 || p.Ls % cfg.spt) return -2;
   switch (op) {
-    case OP_D: return launch_spt<P, OP_D, VAR, true>(p, cfg, st);
+    case OP_D:
+      if constexpr (std::is_same<typename P::C, float>::value)
+        return launch_spt<P, OP_D, VAR, true>(p, cfg, st);
+      return -2;
     case OP_DDAG: return launch_spt<P, OP_DDAG, VAR, true>(p, cfg, st);
     case OP_HOP_LOCAL: return launch_spt<P, OP_HOP_LOCAL, VAR, true>(p, cfg, st);
     case OP_HOP_SCALED_DAG: return launch_spt<P, OP_HOP_SCALED_DAG, VAR, true>(p, cfg, st);

@@ -256,7 +256,12 @@ int launch_m5_p(const M5Params &q, M5Kind kind, cudaStream_t st) {
     case M5_A: m5_kernel<P, false><<<blocks, 256, 0, st>>>(q); break;
     case M5_INV: m5_kernel<P, true><<<blocks, 256, 0, st>>>(q); break;
     case M5_INV_PHI: m5_kernel<P, true, true><<<blocks, 256, 0, st>>>(q); break;
-    case M5_PHI: phi_kernel<P><<<blocks, 256, 0, st>>>(q); break;
+    case M5_PHI:  // FP64 only: elsewhere the hops form phi as they read
+      if constexpr (std::is_same<typename P::C, double>::value) {
+        phi_kernel<P><<<blocks, 256, 0, st>>>(q);
+        break;
+      }
+      return fail(DW_ERR_ARG, "the phi pass is FP64 only");
   }
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? DW_OK : cuda_fail(e, "m5 launch");
@@ -464,8 +469,9 @@ int run_dslash_cb(dw_lattice *lat, int prec, int op, void *out, const void *nbr,
 }
 
 // out_o = Dhat in_o (dag: Dhat^+ in_o) at precision prec; t1, t2: even-parity
-// scratch fields; norm_partials (optional, not dag) receives |out|^2 per CTA;
-// fuse (optional, dag only): the CG residual update in place of storing out.
+// scratch fields (t1 is not touched where schur_fused); norm_partials (optional, not
+// dag) receives |out|^2 per CTA; fuse (optional, dag only): the CG residual update in
+// place of storing out.
 // The (b + cK) of the second hop of Dhat and of the first of Dhat^+ rides in the
 // A^-1 pass, so those two are the plain hopping term: no phi per neighbour, no slice
 // exchange (24^4 x 16 FP32: Dhat and Dhat^+ together 1.09 -> 1.01 ms).
@@ -475,46 +481,43 @@ int apply_schur(dw_lattice *lat, int prec, void *out, const void *in, const doub
   const double alpha = lat->b * (4.0 - lat->M5) + 1.0;
   const double beta = lat->c * (4.0 - lat->M5) - 1.0;
   int rc;
-  // FP32 / FP16: the A^-1 pass rides in the hop before it (the M5 forms) where all slices
-  // of a site fit a CTA; t1 is then not used
-  const bool fused = prec != DW_F64 && m5_fits(lat, prec);
-  if (fused) {
-    const double h = -0.5;
-    if ((rc = run_dslash_cb(lat, prec, dag ? OP_HOP_DAG_M5 : OP_D_M5, t2, in, nullptr, 0, alpha,
-                            beta, h, mf, nrhs, st, gate, gate_stride, nullptr)))
-      return rc;
+  if (schur_fused(lat, prec)) {
+    // t2 as below, the A^-1 pass riding in the hop before it (the M5 forms)
+    rc = run_dslash_cb(lat, prec, dag ? OP_HOP_DAG_M5 : OP_D_M5, t2, in, nullptr, 0, alpha, beta,
+                       -0.5, mf, nrhs, st, gate, gate_stride, nullptr);
+    if (rc) return rc;
+  } else {
+    // t1 = H_eo in (dag: -b/2 Dhop^+ in) on even sites
+    if (dag) {
+      rc = run_dslash_cb(lat, prec, OP_HOP_SCALED_DAG, t1, in, nullptr, 0, 0.0, 0.0, -0.5, mf,
+                         nrhs, st, gate, gate_stride, nullptr);
+    } else if (prec == DW_F64) {  // phi in its own pass (see phi_kernel); out is free until the end
+      if ((rc = apply_phi(lat, prec, out, in, true, mf, nrhs, st, gate, gate_stride))) return rc;
+      rc = run_dslash_cb(lat, prec, OP_HOP_LOCAL, t1, out, nullptr, 0, 0.0, 0.0, -0.5, mf, nrhs,
+                         st, gate, gate_stride, nullptr);
+    } else {
+      rc = run_dslash_cb(lat, prec, OP_D, t1, in, nullptr, 0, 0.0, 0.0, -0.5, mf, nrhs, st, gate,
+                         gate_stride, nullptr);
+    }
+    if (rc) return rc;
+    // t2 = (1 + (c/b) K) A^-1 t1 (dag: the adjoint)
+    rc = apply_m5_inv_phi(lat, prec, t2, t1, mf, nrhs, dag, st, gate, gate_stride);
+    if (rc) return rc;
   }
-  if (dag) {
-    // t1 = -b/2 Dhop^+ in on even sites, t2 = (1 + (c/b) K^+) A^-+ t1
-    if (!fused && ((rc = run_dslash_cb(lat, prec, OP_HOP_SCALED_DAG, t1, in, nullptr, 0, 0.0, 0.0, -0.5, mf,
-                            nrhs, st, gate, gate_stride, nullptr)) ||
-                   (rc = apply_m5_inv_phi(lat, prec, t2, t1, mf, nrhs, true, st, gate,
-                                          gate_stride))))
-      return rc;
-    // out = A^+ in - H_eo^+ t2 on odd sites
+  // out = A in - H_oe A^-1 t1, or A^+ in - H_eo^+ A^-+ t1, on odd sites
+  if (dag)
     return run_dslash_cb(lat, prec, OP_DDAG, out, t2, in, 1, alpha, beta, 0.5, mf, nrhs, st, gate,
                          gate_stride, nullptr, nullptr, fuse);
-  }
-  // t1 = H_eo in on even sites
-  if (prec == DW_F64) {  // phi in its own pass (see phi_kernel); out is free until the end
-    if ((rc = apply_phi(lat, prec, out, in, true, mf, nrhs, st, gate, gate_stride)) ||
-        (rc = run_dslash_cb(lat, prec, OP_HOP_LOCAL, t1, out, nullptr, 0, 0.0, 0.0, -0.5, mf, nrhs,
-                            st, gate, gate_stride, nullptr)))
-      return rc;
-  } else if (!fused && (rc = run_dslash_cb(lat, prec, OP_D, t1, in, nullptr, 0, 0.0, 0.0, -0.5, mf,
-                                           nrhs, st, gate, gate_stride, nullptr))) {
-    return rc;
-  }
-  // t2 = (1 + (c/b) K) A^-1 t1, out = A in - H_oe A^-1 t1 on odd sites
-  if (!fused &&
-      (rc = apply_m5_inv_phi(lat, prec, t2, t1, mf, nrhs, false, st, gate, gate_stride)))
-    return rc;
   return run_dslash_cb(lat, prec, OP_HOP_LOCAL, out, t2, in, 1, alpha, beta, 0.5, mf, nrhs, st,
                        gate, gate_stride, norm_partials);
 }
 
+bool schur_fused(const dw_lattice *lat, int prec) {
+  return prec != DW_F64 && m5_fits(lat, prec);
+}
+
 bool cb_op_used(const dw_lattice *lat, int prec, int op) {
-  const bool fused = prec != DW_F64 && m5_fits(lat, prec);
+  const bool fused = schur_fused(lat, prec);
   switch (op) {
     case OP_D: return prec != DW_F64 && !fused;
     case OP_D_M5:
@@ -661,10 +664,11 @@ extern "C" int dw_apply_schur(dw_lattice *lat, void *out, const void *in, const 
   if (lat->cplx && lat->prec == DW_F32)
     return fail(DW_ERR_STATE, "interleaved-complex FP32 fields support Dhop and Dhop^+ only");
   if ((rc = check_cb(lat, lat->prec, dag != 0))) return rc;
-  const size_t need = 2 * cb_field_bytes(lat, lat->prec, nrhs);
-  if ((rc = ensure_buffer(&lat->scratch, &lat->scratch_bytes, need))) return rc;
-  void *t1 = lat->scratch;
-  void *t2 = (char *)lat->scratch + need / 2;
+  const size_t field = cb_field_bytes(lat, lat->prec, nrhs);
+  const bool fused = schur_fused(lat, lat->prec);
+  if ((rc = ensure_buffer(&lat->scratch, &lat->scratch_bytes, fused ? field : 2 * field))) return rc;
+  void *t2 = lat->scratch;
+  void *t1 = fused ? nullptr : (char *)lat->scratch + field;
   return apply_schur(lat, lat->prec, out, in, mf, nrhs, dag != 0, t1, t2, (cudaStream_t)stream,
                      nullptr, 0, nullptr);
 }
