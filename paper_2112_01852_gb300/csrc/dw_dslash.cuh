@@ -490,8 +490,9 @@ __device__ __forceinline__ void store_spinor(typename P::vec *base, long long pl
 // last and only the last step rounds at size one.  Row error (rms, against FP64 on
 // exp(i eps H) links) at eps 0.03 / 0.3 / 1: 1.7e-8 / 2.5e-8 / 3.8e-8; from the two differences
 // of products 2.4e-8 / 3.1e-8 / 3.8e-8, with a_0 b_1 first 3.4e-8 / 3.9e-8 / 3.8e-8.  The other
-// chains keep their order: with all of them turned round the 32^3 x 64 x 12 Dhop took 1.310 ms
-// at variant 6, 1.243 so.
+// chains keep their order (all of them turned round: 32^3 x 64 x 12 Dhop at variant 6 1.241 ->
+// 1.310 ms), and of the six orders of the small terms this one leaves every stencil its time
+// (D 16^3 x 32 x 12 with 12 RHS 1.520 -> 1.518 ms; the others up to 1.586).
 __device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
 template <class C>
@@ -501,7 +502,7 @@ __device__ __forceinline__ void rebuild_row2(C *U) {
     const int j = (i + 1) % 3, k = (i + 2) % 3;  // row2_i = conj(a_j b_k - a_k b_j)
     const C ajr = U[2 * j], aji = U[2 * j + 1], akr = U[2 * k], aki = U[2 * k + 1];
     const C bjr = U[6 + 2 * j], bji = U[7 + 2 * j], bkr = U[6 + 2 * k], bki = U[7 + 2 * k];
-    U[12 + 2 * i] = i == 2 ? fma_(ajr, bkr, fma_(-akr, bjr, fma_(aki, bji, -aji * bki)))
+    U[12 + 2 * i] = i == 2 ? fma_(ajr, bkr, fma_(aki, bji, fma_(-aji, bki, -akr * bjr)))
                            : fma_(aki, bji, fma_(-akr, bjr, fma_(-aji, bki, ajr * bkr)));
     U[13 + 2 * i] = fma_(aki, bjr, fma_(akr, bji, fma_(-aji, bkr, -ajr * bki)));
   }
