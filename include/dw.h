@@ -105,7 +105,8 @@ int dw_load_gauge(dw_lattice *lat, const void *U, void *stream);
  * out = Dhop in, the bare hopping sum over the 8 neighbours for every slice s
  * and each of nrhs right-hand sides (no -1/2 factor, no diagonal term).
  * This is the paper's Domain Wall kernel (Sec. 4.1; 1320 flop per 5D site,
- * Table 3).
+ * Table 3).  An untuned FP32 or FP16 launch may take the row-staged variant, whose
+ * bounded wait reports through dw_device_status.
  */
 int dw_apply_Dhop(dw_lattice *lat, void *out, const void *in, int nrhs, void *stream);
 /* out = Dhop^+ in  (= g5 Dhop g5 in). */
@@ -113,7 +114,14 @@ int dw_apply_Dhop_dag(dw_lattice *lat, void *out, const void *in, int nrhs, void
 
 /*
  * out = D in with the per-RHS masses mf[nrhs] (HOST array).  One fused pass:
- * (b + cK) is applied to the neighbour spinors before the hop.
+ * (b + cK) is applied to the neighbour spinors before the hop.  At DW_F64 with
+ * nrhs * V4 * Ls >= 2^15 a streaming pass forms (b + cK) in / b first (the same
+ * bits in 0.86 of the time at 16^4 x 16).  It needs one field of device memory,
+ * allocated and freed in stream order from a memory pool that the lattice creates
+ * at its first such call.  The pool keeps the largest single workspace until
+ * dw_destroy_lattice; a cudaMalloc of the process that would fail otherwise is
+ * given that memory.  If there is none to be had, or if `stream` is being
+ * captured, the fused pass runs and nothing is allocated.
  */
 int dw_apply_D(dw_lattice *lat, void *out, const void *in, const double *mf, int nrhs,
                void *stream);
@@ -122,7 +130,8 @@ int dw_apply_Ddag(dw_lattice *lat, void *out, const void *in, const double *mf, 
                   void *stream);
 /*
  * out = D^+ D in.  The intermediate D in lives in lattice-owned scratch, so
- * calls on one lattice must not overlap on different streams.
+ * calls on one lattice must not overlap on different streams.  `out` is scratch
+ * of the D pass too (dw_apply_D's streaming pass) before it holds the result.
  */
 int dw_apply_DdagD(dw_lattice *lat, void *out, const void *in, const double *mf, int nrhs,
                    void *stream);

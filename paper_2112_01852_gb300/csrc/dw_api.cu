@@ -140,7 +140,10 @@ static int largest_divisor(int n, int cap) {
 //  D^+ 1.86 -> 1.76 ms; 10 x 12 x 8 x 20 x 10 D 0.53 -> 0.42).
 // With default_tile's choices within 8 % (FP16 15 %) of the best of all tiles on most of
 // 9^3 x 10 x 5 .. 32^3 x 64 x 12, where one thread row per slice and variant 0 took 1.1 - 2.2
-// times the best.
+// times the best.  A prime Ls splits into CTAs of one warp: at 16 x 16 x 8 x 16 x 11 and 13
+// Dhop takes 26.9 and 32.6 us at FP32 (32.7 and 40.8 with all groups in a CTA), 28.5 and 30.7 at
+// FP16 (32.7, 40.9), 542 at FP64 and 11 (559).  Its D^+ is out of the rule's reach (11 CTAs are
+// no cluster): the general path, 49 and 55 us at FP32 where the tuner finds 43 and 51.
 TileConfig register_tile(const dw_lattice *lat, int prec, int op, int nrhs) {
   const int Ls = lat->Ls;
   // (an Ls that fits no CTA there is refused here too; dw_set_tile and dw_tune split it)
@@ -165,7 +168,9 @@ TileConfig register_tile(const dw_lattice *lat, int prec, int op, int nrhs) {
 //    groups (24^3 x 48 x 8 Dhop 277 -> 262 us);
 //  - D at FP32, and at an odd multiple of three slices: three or four slices per thread
 //    uncapped (variant 2, whose D is the register path: its loads of the s-neighbours
-//    shared by more slices);
+//    shared by more slices).  64 sites wide at an even Ls, but for an odd count of 32-site
+//    blocks below 20, whose last tile stands half empty: 64 against 32 sites take 1.06 - 1.15
+//    times as long at 9 blocks, 1.00 - 1.04 at 13, 0.98 - 1.03 at 17, 0.97 - 1.07 at 21 - 27;
 //  - an odd Ls at FP16, and Dhop at FP64: the prefetch variant 2 (FP64 16^4 x 16 1.65 -> 1.53
 //    ms).
 // All of them sum the hops in the same order: the choice does not change a result.
