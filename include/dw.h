@@ -287,7 +287,7 @@ int dw_solve_eo(dw_lattice *lat, void *x, const void *eta, const double *mf, int
  * at precision `prec` for launches of `nrhs` right-hand sides (0 = any count
  * without a more specific entry).  Returns DW_ERR_ARG for an invalid tile.
  *
- * dw_tune times the untuned tile and a list of valid ones for (op, nrhs) at the
+ * dw_tune times a list of valid tiles and the untuned one for (op, nrhs) at the
  * lattice precision on lattice-owned scratch fields (CUDA events on `stream`,
  * median of a few launches), keeps the fastest for later calls and returns it in *spt, *tx,
  * *variant, *zblk, *sgrp (any may be NULL).  For nrhs > 1 it also chooses the

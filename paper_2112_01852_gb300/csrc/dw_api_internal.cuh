@@ -67,6 +67,10 @@ int ensure_buffer(void **buf, size_t *cap, size_t need);
 TileConfig default_tile(const dw_lattice *lat, int prec, int op, int nrhs);
 TileConfig register_tile(const dw_lattice *lat, int prec, int op, int nrhs);
 TileConfig generic_tile(const dw_lattice *lat, int prec, int op);
+inline bool operator==(const TileConfig &a, const TileConfig &b) {
+  return a.spt == b.spt && a.tx == b.tx && a.variant == b.variant && a.zblk == b.zblk &&
+         a.sgrp == b.sgrp && a.rhs_outer == b.rhs_outer;
+}
 int auto_zblk(const dw_lattice *lat, int prec);
 TileConfig pick_tile(dw_lattice *lat, int prec, int op, int nrhs);
 bool tile_valid(const dw_lattice *lat, int prec, int op, TileConfig t);

@@ -526,7 +526,7 @@ bool cb_op_used(const dw_lattice *lat, int prec, int op) {
   return op == OP_DDAG || op == OP_HOP_LOCAL;
 }
 
-// Times the untuned checkerboard tile of (prec, op) and a list of others on two scratch
+// Times a list of checkerboard tiles of (prec, op) and the untuned one on two scratch
 // parity fields (the hopping-only form, one RHS) and keeps the fastest for later launches.
 int tune_cb(dw_lattice *lat, int prec, int op, cudaStream_t st) {
   if (lat->tuned.count(std::make_tuple(prec, kCbOpKey + op, 0))) return DW_OK;
@@ -550,12 +550,15 @@ int tune_cb(dw_lattice *lat, int prec, int op, cudaStream_t st) {
     return run_dslash_cb(lat, prec, o, lat->stage_out, lat->stage_in, nullptr, 0, 4.0, 0.5, -0.5,
                          &mf, 1, st, nullptr, 0, nullptr, &t);
   };
-  // the faster of two launches (1e30: the tile does not launch)
-  auto time_tile = [&](const TileConfig &t) {
+  const TileConfig untuned = cb_default_tile(lat, prec, op);
+  TileConfig best_t = untuned;
+  float best = 1e30f;
+  // takes the tile if the faster of two launches beats `best`
+  auto try_tile = [&](const TileConfig &t) {
     float best_ms = 1e30f;
-    if (launch(op, t) || (op == OP_HOP_LOCAL && launch(OP_HOP_SCALED_DAG, t))) {
+    if (launch(op, t)) {
       cudaGetLastError();
-      return best_ms;  // CTA limits (of either hop that runs on this tile, see cb_tile)
+      return;  // CTA limits
     }
     for (int r = 0; r < 2; ++r) {
       cudaEventRecord(e0, st);
@@ -565,12 +568,16 @@ int tune_cb(dw_lattice *lat, int prec, int op, cudaStream_t st) {
       float m = 1e30f;
       if (cudaEventElapsedTime(&m, e0, e1) == cudaSuccess) best_ms = std::min(best_ms, m);
     }
-    return best_ms;
+    if (best_ms >= best) return;
+    // the limits of the other hop that runs on this tile (see cb_tile)
+    if (op == OP_HOP_LOCAL && launch(OP_HOP_SCALED_DAG, t)) {
+      cudaGetLastError();
+      return;
+    }
+    best = best_ms;
+    best_t = t;
   };
-  // the untuned tile is the one to beat: its slice groups need not be in the list below
-  const TileConfig untuned = cb_default_tile(lat, prec, op);
-  TileConfig best_t = untuned;
-  float best = time_tile(best_t);
+  bool listed = false;  // the untuned tile is in the list
   const int za = auto_zblk(lat, prec);
   for (int spt : {1, 2, 3, 4})
     for (int tx : {32, 64, 96, 128})
@@ -579,14 +586,11 @@ int tune_cb(dw_lattice *lat, int prec, int op, cudaStream_t st) {
         if ((op == OP_D_M5 || op == OP_HOP_DAG_M5) && (tx > 64 || sgrp > 1)) continue;
         const TileConfig t{spt, tx, prec == DW_F64 ? 0 : 4, za, sgrp};
         if (tx * (lat->Ls / spt / sgrp) > 1024) continue;
-        const float ms = time_tile(t);
-        if (ms < best) {
-          best = ms;
-          best_t = t;
-        }
+        listed |= t == untuned;
+        try_tile(t);
       }
-  // again beside the winner: the first timing may have met rising clocks
-  if (time_tile(untuned) <= time_tile(best_t)) best_t = untuned;
+  // the untuned tile is the one to beat, also where its slice groups are not in the list
+  if (!listed) try_tile(untuned);
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   clear_error();

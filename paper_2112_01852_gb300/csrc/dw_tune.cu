@@ -1,5 +1,5 @@
-// Tile autotuner for the stencil kernel: times the untuned tile and every valid tile of a
-// list on lattice-owned scratch fields with CUDA events and keeps the fastest.
+// Tile autotuner for the stencil kernel: times every valid tile of a list and the untuned
+// tile on lattice-owned scratch fields with CUDA events and keeps the fastest.
 #include <algorithm>
 #include <vector>
 
@@ -48,10 +48,10 @@ int tune_tile(dw_lattice *lat, int prec, int op, int nrhs, cudaStream_t st, bool
     std::sort(ms.begin(), ms.end());
     return ms[ms.size() / 2];
   };
-  // the untuned tile is the one to beat: its slice groups need not be in the list below
   const TileConfig untuned = default_tile(lat, prec, op, nrhs);
   TileConfig best_t = untuned;
-  float best = time_tile(best_t);
+  float best = 1e30f;
+  bool listed = false;  // the untuned tile is in the list
   // z-blockings: unblocked, the automatic one and twice that (quick: automatic)
   const int za = auto_zblk(lat, prec);
   std::vector<int> zbs{za};
@@ -68,14 +68,15 @@ int tune_tile(dw_lattice *lat, int prec, int op, int nrhs, cudaStream_t st, bool
               const TileConfig t{spt, tx, variant, zblk, sgrp, outer};
               if (quick && tx > 128) continue;
               if (!tile_valid(lat, prec, op, t)) continue;
+              listed |= t == untuned;
               const float ms = time_tile(t);
               if (ms < best) {
                 best = ms;
                 best_t = t;
               }
             }
-  // again beside the winner: the first timing may have met rising clocks
-  if (time_tile(untuned) <= time_tile(best_t)) best_t = untuned;
+  // the untuned tile is the one to beat, also where its slice groups are not in the list
+  if (!listed && time_tile(untuned) <= best) best_t = untuned;
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   clear_error();

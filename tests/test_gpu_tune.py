@@ -1,4 +1,4 @@
-"""The tuners start from the untuned tile: what they keep is not slower than it, also where
+"""The tuners time the untuned tile too: what they keep is not slower than it, also where
 the rule's slice groups (5, 7, 13 of them here) are not in the list that they try."""
 
 import numpy as np
