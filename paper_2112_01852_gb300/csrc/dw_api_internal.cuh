@@ -96,8 +96,9 @@ int run_dslash(dw_lattice *lat, int prec, int op, void *out, const void *in,
                int t_count = 0, const ResidualFuse *fuse = nullptr, void *phi = nullptr);
 // Scratch of one call on `st`, from the lattice's pool (stream-ordered: allocated and
 // freed on the stream; the pool keeps the largest single block for the next call, memory
-// that the driver hands to a cudaMalloc that would fail).  Null, and no error, where there is none to be had: on a
-// capturing stream, out of memory, or for a call that gains nothing from it.
+// that the driver hands to a cudaMalloc that would fail).  Null, and no error, where there
+// is none to be had: on a capturing stream, out of memory, or for a call that gains
+// nothing from it.
 struct PhiScratch {
   void *p = nullptr;
   cudaStream_t st;

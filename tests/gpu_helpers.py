@@ -98,7 +98,7 @@ def launches(f, name):
             torch.cuda.synchronize()
         return [e.name for e in p.events()]
 
-    for _ in range(3):  # a process's first profile can come back empty
+    for _ in range(10):  # a process's first profile can come back empty
         if profile(lambda: torch.zeros(8, device="cuda").add_(1)):
             break
     return sum(name in n for n in profile(f))
